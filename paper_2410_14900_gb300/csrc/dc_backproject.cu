@@ -1122,6 +1122,20 @@ BPArgs bp_args(const dc_geometry *g, int B, const void *gF, int dtype, const flo
 
 namespace dc {
 
+bool encode_map_f32(CUtensorMap *m, const void *base, size_t d0, size_t d1, size_t d2, int b0,
+                    int b1) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {d0, d1, d2};
+  cuuint64_t strides[2] = {d0 * sizeof(float), d0 * d1 * sizeof(float)};
+  cuuint32_t box[3] = {(cuuint32_t)b0, (cuuint32_t)b1, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int backproject_check(const dc_geometry *g, int B, const void *gF, int dtype,
                       const float *gF_scale, const float *vol, unsigned flags, const char *who) {
   int rc = check_bp(g, B, who);

@@ -2,6 +2,7 @@
 // Defrise-Clack library (handle layout, error plumbing, small device helpers).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cstddef>
 #include <cstdint>
@@ -153,6 +154,12 @@ struct dc_geometry {
   size_t sino_stride;        // floats per padded sinogram (n_mu * NSp)
   int Wp, NSp;               // padded row lengths (multiples of 4)
   int ls_rb;                 // line-sum band height (32, 16 or 8 rows)
+  // line sums of four images at once (every view has the same principal point)
+  int quad;                  // 1 if the geometry and its shared memory allow it
+  int q_mg, q_n_groups;      // max angles per group, groups
+  dc::MuGroup *q_groups;     // [q_n_groups]
+  float *w_imgT;             // [chunk / 4][W][H][4] (w_img holds [chunk / 4][H][W][4])
+  CUtensorMap q_tm_cols, q_tm_rows;  // over w_imgT and w_img
   float *w_img;              // [chunk][H][Wp]
   float *w_sinoA;            // [chunk][n_mu][NSp]
   float *w_sinoB;            // [chunk][n_mu][NSp]
@@ -166,9 +173,16 @@ struct dc_geometry {
 
 namespace dc {
 
+// tiled tensor map over a dense [d2][d1][d0] FP32 array (d0 a multiple of 4),
+// box b0 x b1 x 1, zero fill outside; false if the driver has no encoder
+bool encode_map_f32(CUtensorMap *m, const void *base, size_t d0, size_t d1, size_t d2, int b0,
+                    int b1);
+
 // host-side helpers defined in dc_filter.cu / dc_backproject.cu
 int alloc_workspace(dc_geometry *g);
 int build_mu_tables(dc_geometry *g);
+// whether the four-image line sums apply (g->quad) and their angles per group
+int quad_plan(dc_geometry *g);
 // argument checks of the filter entry points (DC_OK or the error code)
 int filter_check(const dc_geometry *g, int B, const float *gin, const void *gF, int dtype,
                  const float *gF_scale, const char *who);

@@ -14,7 +14,8 @@
 //               the band step as the fastest index; neighbouring lines of a
 //               warp take the s-difference by shuffle so that D_f never
 //               subtracts two large sums; the epilogue applies w_sino, K, W
-//               and D_b (or the adjoint chain)
+//               and D_b (or the adjoint chain); four images at once where
+//               every view has the same principal point (k_linesum4)
 //   k_bp2d      pixel-driven A2d^T: each pixel gathers the two sinogram taps
 //               of every angle (the exact transpose of the Joseph weights),
 //               angles streamed through shared memory with bulk copies; the
@@ -409,6 +410,8 @@ __device__ __forceinline__ void linesum_body(const LineArgs &a, int gi, int n, i
     }
   }
 }
+
+#include "dc_filter_quad.cuh"
 
 template <int MODE, int RB>
 __global__ void __launch_bounds__(LS_THREADS, 1) k_linesum(LineArgs a) {
@@ -882,7 +885,26 @@ size_t bp2d_smem(const dc_geometry *g) {
 }
 
 template <int MODE>
-int launch_linesum(const dc_geometry *g, LineArgs &a, cudaStream_t st) {
+int launch_linesum4(const dc_geometry *g, LineArgs &a, cudaStream_t st) {
+  const L4Shape sh = l4_shape(a.H, a.W);
+  a.mg = g->q_mg;
+  a.groups = g->q_groups;
+  DC_CUDA(cudaFuncSetAttribute(k_linesum4<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               L4_SMEM_BUDGET));
+  dim3 grid(g->q_n_groups, (a.n_img + 3) / 4);
+  k_linesum4<MODE><<<grid, L4_THREADS, l4_smem(sh, a.mg, a.NSp), st>>>(a, sh, g->q_tm_cols,
+                                                                       g->q_tm_rows);
+  DC_CHECK_LAUNCH("k_linesum4");
+  return DC_OK;
+}
+
+// line sums of the images that launch_prep staged with the same `quad`
+template <int MODE>
+int launch_linesum(const dc_geometry *g, LineArgs &a, bool quad, cudaStream_t st) {
+  if (quad) {
+    dc::ProfScope ps(dc::KID_LINESUM, st);
+    return launch_linesum4<MODE>(g, a, st);
+  }
   size_t sm = linesum_smem(g);
   dim3 grid(g->n_groups, a.n_img);
   dc::ProfScope ps(dc::KID_LINESUM, st);
@@ -916,7 +938,7 @@ int launch_bp2d(const dc_geometry *g, BP2Args &a, cudaStream_t st) {
 }
 
 int launch_prep(const dc_geometry *g, const float *src, int weight, int v0, int n_img, int B,
-                int b0, cudaStream_t st) {
+                int b0, bool quad, cudaStream_t st) {
   const dc_geometry_desc &d = g->d;
   PrepArgs p;
   p.src = src;
@@ -933,8 +955,14 @@ int launch_prep(const dc_geometry *g, const float *src, int weight, int v0, int 
   p.n_img = n_img;
   p.pitch = (float)d.pitch;
   p.weight = weight;
-  dim3 grid((g->Wp + 31) / 32, (d.det_rows + 31) / 32, n_img);
   dc::ProfScope ps(dc::KID_PREP, st);
+  if (quad) {
+    dim3 grid((d.det_cols + 31) / 32, (d.det_rows + 31) / 32, (n_img + 3) / 4);
+    k_prep4<<<grid, dim3(32, 8), 0, st>>>(p, (float4 *)g->w_img, (float4 *)g->w_imgT);
+    DC_CHECK_LAUNCH("k_prep4");
+    return DC_OK;
+  }
+  dim3 grid((g->Wp + 31) / 32, (d.det_rows + 31) / 32, n_img);
   k_prep<<<grid, dim3(32, 8), 0, st>>>(p);
   DC_CHECK_LAUNCH("k_prep");
   return DC_OK;
@@ -1016,6 +1044,12 @@ Chunking chunking(const dc_geometry *g, int B, int view_limit = 0) {
   if (view_limit > 0) c.cv = std::min(c.cv, view_limit);
   return c;
 }
+
+// Four images at once cost about the time of two single ones (their step
+// runs at more than twice the rate), so single-image chunks keep the
+// per-image kernel.  The rule looks at the plan of the whole call, not at a
+// chunk, so that every image of a call takes the same path.
+bool use_quad(const dc_geometry *g, int bc, int cv) { return g->quad && bc * cv >= 2; }
 
 // ------------------------------------------------ batched persistent filter
 // One kernel filters every view of a batch of problems (orbits with uneven
@@ -1168,20 +1202,54 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 
 namespace dc {
 
+// The four-image line sums share every sample position, so all views need
+// the same principal point.  Matrices of one scanner give it up to the
+// rounding of their recovery (~1e-10 pixels); 1e-8 pixels is below a
+// hundredth of the FP32 positions' own rounding (~1e-6), and a detector
+// calibrated view by view differs by far more and keeps the per-image
+// kernel, as do rows too long for two stages.  The angles per group are the
+// number with the least time per angle: rounds of a CTA's warps over its
+// tasks, plus half a round for set-up and epilogue.
+int quad_plan(dc_geometry *g) {
+  const dc_geometry_desc &d = g->d;
+  g->quad = 0;
+  if (getenv("DC_NO_QUAD") || d.det_rows < L4_RB || d.det_cols < L4_RB) return DC_OK;
+  for (int i = 1; i < d.n_views; ++i)
+    for (int c = 13; c <= 14; ++c)
+      if (!(std::fabs(g->host_geo[(size_t)DC_VIEW_GEO_N * i + c] - g->host_geo[c]) < 1e-8))
+        return DC_OK;
+  const int nch = (d.n_s + 31) / 32, NSp = round4(d.n_s);
+  const L4Shape sh = l4_shape(d.det_rows, d.det_cols);
+  double best = 0.0;
+  for (int mg = 1; mg <= DC_LS_MAX_MG && mg * nch <= L4_TASKS; ++mg) {
+    if (l4_smem(sh, mg, NSp) > L4_SMEM_BUDGET) break;
+    const double cost = ((mg * nch + L4_WARPS - 1) / L4_WARPS + 0.5) / mg;
+    if (!g->quad || cost < best) {
+      best = cost;
+      g->q_mg = mg;
+      g->quad = 1;
+    }
+  }
+  return DC_OK;
+}
+
 int alloc_workspace(dc_geometry *g) {
   const dc_geometry_desc &d = g->d;
   g->Wp = round4(d.det_cols);
   g->NSp = round4(d.n_s);
   g->img_stride = (size_t)d.det_rows * g->Wp;
   g->sino_stride = (size_t)d.n_mu * g->NSp;
-  size_t per_img = (g->img_stride + 2 * g->sino_stride) * sizeof(float);
-  // size the work area near 112 MB (resident in the 126 MB L2); the
-  // autotuner may use fewer images per chunk than it holds
-  long target = 112L << 20;
+  size_t per_img = ((g->quad ? 2 : 1) * g->img_stride + 2 * g->sino_stride) * sizeof(float);
+  // The per-image kernels want a chunk that stays in the 126 MB L2 (112 MB);
+  // the four-image kernels take few CTAs per image, so larger chunks keep the
+  // last wave of a launch small (their L2 working set is the few images in
+  // flight).  The autotuner may use fewer images per chunk than it holds.
+  long target = (g->quad ? 384L : 112L) << 20;
   const char *env = getenv("DC_CHUNK_IMAGES");
   int ci = env ? atoi(env) : (int)(target / (long)per_img);
   if (ci < 4) ci = 4;
   if (ci > 256) ci = 256;
+  if (g->quad) ci &= ~3;
   g->chunk_images = ci;
   g->chunk_capacity = ci;
   g->bp_nz = 32;
@@ -1189,6 +1257,14 @@ int alloc_workspace(dc_geometry *g) {
   if (g->ls_rb == 0 || bp2d_smem(g) > 200 * 1024)
     return fail(DC_ERR_UNSUPPORTED, "detector or sinogram rows too long for shared memory");
   DC_CUDA(dmalloc((void **)&g->w_img, sizeof(float) * g->img_stride * ci));
+  if (g->quad) {
+    const size_t H = d.det_rows, W = d.det_cols, ng = ci / 4;
+    const L4Shape sh = l4_shape(d.det_rows, d.det_cols);
+    DC_CUDA(dmalloc((void **)&g->w_imgT, sizeof(float) * 4 * H * W * ng));
+    if (!encode_map_f32(&g->q_tm_cols, g->w_imgT, 4 * H, W, ng, 4 * L4_RB, sh.boxh[0]) ||
+        !encode_map_f32(&g->q_tm_rows, g->w_img, 4 * W, H, ng, 4 * L4_RB, sh.boxh[1]))
+      g->quad = 0;
+  }
   DC_CUDA(dmalloc((void **)&g->w_sinoA, sizeof(float) * g->sino_stride * ci));
   DC_CUDA(dmalloc((void **)&g->w_sinoB, sizeof(float) * g->sino_stride * ci));
   DC_CUDA(dmalloc((void **)&g->w_absmax, sizeof(unsigned) * ci));
@@ -1226,12 +1302,13 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
   const dc_geometry_desc &d = g->d;
   const int n_img = nv * bc;
   int rc;
-  if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, st))) return rc;
+  const bool quad = use_quad(g, g->chunk_images, 1);
+  if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, quad, st))) return rc;
   LineArgs la = line_args(g, bc, v0, b0, n_img);
   la.Wred = W;
   la.out = g->w_sinoA;
   la.Sout = S;
-  if ((rc = launch_linesum<M_FILTER>(g, la, st))) return rc;
+  if ((rc = launch_linesum<M_FILTER>(g, la, quad, st))) return rc;
   BP2Args ba = bp2_args(g, bc, v0, b0, n_img, g->w_sinoA);
   ba.weight = WT_D;
   if (dtype == DC_F16) {
@@ -1446,21 +1523,22 @@ int dc_filter_adjoint(const dc_geometry *g, int B, const float *grad_gF, const f
   if (!grad_g && !grad_W) return DC_OK;
   cudaStream_t st = (cudaStream_t)stream;
   Chunking ck = chunking(g, B, view_chunk);
+  const bool quad = use_quad(g, ck.bc, ck.cv);
   for (int b0 = 0; b0 < B; b0 += ck.bc) {
     int bc = std::min(ck.bc, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += ck.cv) {
       int nv = std::min(ck.cv, d.n_views - v0);
       int n_img = nv * bc;
       // dL/dP up to D_b^T: line differences of w_d * dL/dg^F
-      if ((rc = launch_prep(g, grad_gF, WT_D, v0, n_img, bc, b0, st))) return rc;
+      if ((rc = launch_prep(g, grad_gF, WT_D, v0, n_img, bc, b0, quad, st))) return rc;
       LineArgs la = line_args(g, bc, v0, b0, n_img);
       la.Wred = W;
       la.sinoA = g->w_sinoA;
       la.sinoB = g->w_sinoB;
-      if ((rc = launch_linesum<M_DIFFSTORE>(g, la, st))) return rc;
+      if ((rc = launch_linesum<M_DIFFSTORE>(g, la, quad, st))) return rc;
       // recompute S from w_cos * g and finish the chain
-      if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, st))) return rc;
-      if ((rc = launch_linesum<M_ADJ>(g, la, st))) return rc;
+      if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, quad, st))) return rc;
+      if ((rc = launch_linesum<M_ADJ>(g, la, quad, st))) return rc;
       if (grad_W) {
         size_t total = (size_t)nv * d.n_mu * d.n_s;
         int nb = (int)std::min<size_t>((total + 255) / 256, 4096);
@@ -1495,18 +1573,19 @@ int dc_filter_adjoint_from_s(const dc_geometry *g, int B, const float *grad_gF,
   if (!grad_g && !grad_W) return DC_OK;
   cudaStream_t st = (cudaStream_t)stream;
   Chunking ck = chunking(g, B, view_chunk);
+  const bool quad = use_quad(g, ck.bc, ck.cv);
   for (int b0 = 0; b0 < B; b0 += ck.bc) {
     int bc = std::min(ck.bc, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += ck.cv) {
       int nv = std::min(ck.cv, d.n_views - v0);
       int n_img = nv * bc;
       // dL/dP up to D_b^T: line differences of w_d * dL/dg^F
-      if ((rc = launch_prep(g, grad_gF, WT_D, v0, n_img, bc, b0, st))) return rc;
+      if ((rc = launch_prep(g, grad_gF, WT_D, v0, n_img, bc, b0, quad, st))) return rc;
       LineArgs la = line_args(g, bc, v0, b0, n_img);
       la.Wred = W;
       la.sinoA = g->w_sinoA;
       la.sinoB = g->w_sinoB;
-      if ((rc = launch_linesum<M_DIFFSTORE>(g, la, st))) return rc;
+      if ((rc = launch_linesum<M_DIFFSTORE>(g, la, quad, st))) return rc;
       {  // finish the chain with the stored S
         dim3 grid((d.n_mu + AS_ROWS - 1) / AS_ROWS, n_img);
         dc::ProfScope ps(dc::KID_ADJ_S, st);
@@ -1540,14 +1619,15 @@ int dc_grangeat(const dc_geometry *g, int B, const float *gin, float *S, void *s
   const dc_geometry_desc &d = g->d;
   cudaStream_t st = (cudaStream_t)stream;
   Chunking ck = chunking(g, B);
+  const bool quad = use_quad(g, ck.bc, ck.cv);
   for (int b0 = 0; b0 < B; b0 += ck.bc) {
     int bc = std::min(ck.bc, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += ck.cv) {
       int n_img = std::min(ck.cv, d.n_views - v0) * bc;
-      if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, st))) return rc;
+      if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, quad, st))) return rc;
       LineArgs la = line_args(g, bc, v0, b0, n_img);
       la.out = S;
-      if ((rc = launch_linesum<M_GRANGEAT>(g, la, st))) return rc;
+      if ((rc = launch_linesum<M_GRANGEAT>(g, la, quad, st))) return rc;
     }
   }
   return DC_OK;
@@ -1560,14 +1640,15 @@ int dc_radon2d(const dc_geometry *g, int B, const float *img, float *R, void *st
   const dc_geometry_desc &d = g->d;
   cudaStream_t st = (cudaStream_t)stream;
   Chunking ck = chunking(g, B);
+  const bool quad = use_quad(g, ck.bc, ck.cv);
   for (int b0 = 0; b0 < B; b0 += ck.bc) {
     int bc = std::min(ck.bc, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += ck.cv) {
       int n_img = std::min(ck.cv, d.n_views - v0) * bc;
-      if ((rc = launch_prep(g, img, WT_NONE, v0, n_img, bc, b0, st))) return rc;
+      if ((rc = launch_prep(g, img, WT_NONE, v0, n_img, bc, b0, quad, st))) return rc;
       LineArgs la = line_args(g, bc, v0, b0, n_img);
       la.out = R;
-      if ((rc = launch_linesum<M_RAW>(g, la, st))) return rc;
+      if ((rc = launch_linesum<M_RAW>(g, la, quad, st))) return rc;
     }
   }
   return DC_OK;

@@ -160,6 +160,8 @@ void free_geometry(dc_geometry *g) {
   cudaFree(g->vmu);
   cudaFree(g->mu_order);
   cudaFree(g->groups);
+  cudaFree(g->q_groups);
+  cudaFree(g->w_imgT);
   cudaFree(g->w_img);
   cudaFree(g->w_sinoA);
   cudaFree(g->w_sinoB);
@@ -207,6 +209,29 @@ int build_mu_tables(dc_geometry *g) {
       groups.push_back(G);
     }
     if (br == 0) g->n_groups_branch0 = (int)groups.size();
+  }
+  // the groups of the four-image line sums, over the same order: as even as
+  // the group size allows
+  int rc = quad_plan(g);
+  if (rc) return rc;
+  std::vector<MuGroup> qgroups;
+  for (int br = 0; br < 2 && g->quad; ++br) {
+    const int n = (int)(br ? b1.size() : b0.size()), base = br ? (int)b0.size() : 0;
+    const int ng = (n + g->q_mg - 1) / g->q_mg;
+    for (int t = 0; t < ng; ++t) {
+      MuGroup G;
+      G.first = base + (int)((long long)n * t / ng);
+      G.count = base + (int)((long long)n * (t + 1) / ng) - G.first;
+      G.branch = br;
+      G.pad = 0;
+      qgroups.push_back(G);
+    }
+  }
+  g->q_n_groups = (int)qgroups.size();
+  if (g->quad) {
+    DC_CUDA(dmalloc((void **)&g->q_groups, sizeof(MuGroup) * qgroups.size()));
+    DC_CUDA(cudaMemcpy(g->q_groups, qgroups.data(), sizeof(MuGroup) * qgroups.size(),
+                       cudaMemcpyHostToDevice));
   }
   g->n_groups = (int)groups.size();
   DC_CUDA(dmalloc((void **)&g->mu, sizeof(MuRec) * n_mu));
