@@ -154,12 +154,16 @@ struct dc_geometry {
   size_t sino_stride;        // floats per padded sinogram (n_mu * NSp)
   int Wp, NSp;               // padded row lengths (multiples of 4)
   int ls_rb;                 // line-sum band height (32, 16 or 8 rows)
-  // line sums of four images at once (every view has the same principal point)
+  // line sums and 2-D backprojection of four images at once (every view has the same principal point)
   int quad;                  // 1 if the geometry and its shared memory allow it
   int q_mg, q_n_groups;      // max angles per group, groups
   dc::MuGroup *q_groups;     // [q_n_groups]
   float *w_imgT;             // [chunk / 4][W][H][4] (w_img holds [chunk / 4][H][W][4])
   CUtensorMap q_tm_cols, q_tm_rows;  // over w_imgT and w_img
+  // quad sinograms (w_sinoA, w_sinoB as [chunk / 4][n_mu][NSp][4]): the
+  // s-windows of the 2-D backprojection's tiles of q_ry rows per thread
+  CUtensorMap q_tm_sinoA, q_tm_sinoB;
+  int q_ry;
   float *w_img;              // [chunk][H][Wp]
   float *w_sinoA;            // [chunk][n_mu][NSp]
   float *w_sinoB;            // [chunk][n_mu][NSp]

@@ -411,8 +411,6 @@ __device__ __forceinline__ void linesum_body(const LineArgs &a, int gi, int n, i
   }
 }
 
-#include "dc_filter_quad.cuh"
-
 template <int MODE, int RB>
 __global__ void __launch_bounds__(LS_THREADS, 1) k_linesum(LineArgs a) {
   extern __shared__ __align__(16) float smem[];
@@ -696,6 +694,8 @@ __device__ __forceinline__ bool bp2d_tile(const BP2Args &a, int n, int slot, int
   return true;
 }
 
+#include "dc_filter_quad.cuh"
+
 template <bool MULTI>
 __global__ void __launch_bounds__(BP2_THREADS) k_bp2d(BP2Args a) {
   extern __shared__ __align__(16) float smem[];
@@ -766,7 +766,9 @@ __global__ void k_to_pairs(const float *__restrict__ src, int H, int W, int Wp, 
   }
 }
 
-// sum over the batch of the per-image dL/dW contributions (fixed order)
+// sum over the batch of the per-image dL/dW contributions (fixed order);
+// QUAD: the images are interleaved by four
+template <bool QUAD>
 __global__ void k_reduce_gradW(const float *__restrict__ sinoA, int n_mu, int n_s, int NSp,
                                int B, int v0, int nv, int accumulate,
                                float *__restrict__ gradW) {
@@ -778,7 +780,11 @@ __global__ void k_reduce_gradW(const float *__restrict__ sinoA, int n_mu, int n_
     int m = (int)(t % n_mu);
     int vl = (int)(t / n_mu);
     float s = 0.0f;
-    for (int b = 0; b < B; ++b) s += sinoA[(((size_t)vl * B + b) * n_mu + m) * NSp + k];
+    for (int b = 0; b < B; ++b) {
+      const size_t n = (size_t)vl * B + b;
+      s += QUAD ? sinoA[(((n >> 2) * n_mu + m) * NSp + k) * 4 + (n & 3)]
+                : sinoA[(n * n_mu + m) * NSp + k];
+    }
     size_t o = ((size_t)(v0 + vl) * n_mu + m) * n_s + k;
     gradW[o] = accumulate ? gradW[o] + s : s;
   }
@@ -917,7 +923,37 @@ int launch_linesum(const dc_geometry *g, LineArgs &a, bool quad, cudaStream_t st
 
 bool multi_tap(const dc_geometry *g) { return g->d.ds < g->d.pitch * (1.0 - 1e-12); }
 
-int launch_bp2d(const dc_geometry *g, BP2Args &a, cudaStream_t st) {
+template <int NT, int RY>
+int launch_bp2d4_t(const dc_geometry *g, BP2Args &a, const B4Shape &sh, const CUtensorMap &tm,
+                   cudaStream_t st) {
+  const size_t sm = (size_t)2 * B4_MC * sh.lwb * sh.nb * 16;
+  DC_CUDA(cudaFuncSetAttribute(k_bp2d4<NT, RY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sm));
+  const int tx = 32 * sh.nwx, ty = RY * (8 / sh.nwx);
+  dim3 grid((a.W + tx - 1) / tx, (a.H + ty - 1) / ty, (a.n_img + 3) / 4);
+  k_bp2d4<NT, RY><<<grid, B4_THREADS, sm, st>>>(a, sh, tm);
+  DC_CHECK_LAUNCH("k_bp2d4");
+  return DC_OK;
+}
+
+template <int NT>
+int launch_bp2d4(const dc_geometry *g, BP2Args &a, cudaStream_t st) {
+  const B4Shape sh = b4_shape(a.H, a.W, g->d.pitch, g->d.ds, g->q_ry);
+  const CUtensorMap &tm = (a.sino == g->w_sinoB) ? g->q_tm_sinoB : g->q_tm_sinoA;
+  return g->q_ry == 2 ? launch_bp2d4_t<NT, 2>(g, a, sh, tm, st)
+                      : launch_bp2d4_t<NT, 8>(g, a, sh, tm, st);
+}
+
+// 2-D backprojection of the sinograms that the same `quad` laid out
+int launch_bp2d(const dc_geometry *g, BP2Args &a, bool quad, cudaStream_t st) {
+  if (quad) {
+    dc::ProfScope ps(dc::KID_BP2D, st);
+    switch (b4_taps(g->d.pitch, g->d.ds)) {
+      case 2: return launch_bp2d4<2>(g, a, st);
+      case 4: return launch_bp2d4<4>(g, a, st);
+      default: return launch_bp2d4<6>(g, a, st);
+    }
+  }
   size_t sm = bp2d_smem(g);
   static bool attr_done = false;
   if (!attr_done) {
@@ -1267,6 +1303,14 @@ int alloc_workspace(dc_geometry *g) {
   }
   DC_CUDA(dmalloc((void **)&g->w_sinoA, sizeof(float) * g->sino_stride * ci));
   DC_CUDA(dmalloc((void **)&g->w_sinoB, sizeof(float) * g->sino_stride * ci));
+  if (g->quad) {
+    const size_t ng = ci / 4, n0 = 4 * (size_t)g->NSp, n1 = d.n_mu;
+    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, std::min(d.n_views, ci));
+    const int lwb = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry).lwb;
+    if (!encode_map_f32(&g->q_tm_sinoA, g->w_sinoA, n0, n1, ng, 4 * lwb, 1) ||
+        !encode_map_f32(&g->q_tm_sinoB, g->w_sinoB, n0, n1, ng, 4 * lwb, 1))
+      g->quad = 0;
+  }
   DC_CUDA(dmalloc((void **)&g->w_absmax, sizeof(unsigned) * ci));
   DC_CUDA(dmalloc((void **)&g->w_flags, sizeof(unsigned) * 4));
   DC_CUDA(cudaMemset(g->w_flags, 0, sizeof(unsigned) * 4));
@@ -1315,7 +1359,7 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
     DC_CUDA(cudaMemsetAsync(g->w_absmax, 0, sizeof(unsigned) * n_img, st));
     ba.out_kind = OUT_F32_ABSMAX;
     ba.out = g->w_img;
-    if ((rc = launch_bp2d(g, ba, st))) return rc;
+    if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
     dim3 grid(64, n_img);
     ProfScope ps(KID_TO_F16, st);
     k_to_f16<<<grid, 256, 0, st>>>(g->w_img, g->w_absmax, d.det_rows, d.det_cols, g->Wp,
@@ -1325,7 +1369,7 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
     // g^F of the chunk into the work area (L2-resident), then the pairs
     ba.out_kind = OUT_F32_SLOT;
     ba.out = g->w_img;
-    if ((rc = launch_bp2d(g, ba, st))) return rc;
+    if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
     const int pairs_per_img = d.det_rows * ((d.det_cols + 1) / 2);
     dim3 grid((unsigned)std::min(64, (pairs_per_img + 255) / 256), n_img);
     ProfScope ps(KID_TO_PAIRS, st);
@@ -1335,7 +1379,7 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
   } else {
     ba.out_kind = (dtype == DC_BF16) ? OUT_BF16 : OUT_F32;
     ba.out = gF;
-    if ((rc = launch_bp2d(g, ba, st))) return rc;
+    if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
   }
   return DC_OK;
 }
@@ -1543,8 +1587,8 @@ int dc_filter_adjoint(const dc_geometry *g, int B, const float *grad_gF, const f
         size_t total = (size_t)nv * d.n_mu * d.n_s;
         int nb = (int)std::min<size_t>((total + 255) / 256, 4096);
         dc::ProfScope ps(dc::KID_REDUCE_W, st);
-        k_reduce_gradW<<<nb, 256, 0, st>>>(g->w_sinoA, d.n_mu, d.n_s, g->NSp, bc, v0, nv,
-                                           b0 > 0, grad_W);
+        auto reduce = quad ? k_reduce_gradW<true> : k_reduce_gradW<false>;
+        reduce<<<nb, 256, 0, st>>>(g->w_sinoA, d.n_mu, d.n_s, g->NSp, bc, v0, nv, b0 > 0, grad_W);
         DC_CHECK_LAUNCH("k_reduce_gradW");
       }
       if (grad_g) {
@@ -1552,7 +1596,7 @@ int dc_filter_adjoint(const dc_geometry *g, int B, const float *grad_gF, const f
         ba.weight = WT_COS;
         ba.out_kind = OUT_F32;
         ba.out = grad_g;
-        if ((rc = launch_bp2d(g, ba, st))) return rc;
+        if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
       }
     }
   }
@@ -1587,17 +1631,24 @@ int dc_filter_adjoint_from_s(const dc_geometry *g, int B, const float *grad_gF,
       la.sinoB = g->w_sinoB;
       if ((rc = launch_linesum<M_DIFFSTORE>(g, la, quad, st))) return rc;
       {  // finish the chain with the stored S
-        dim3 grid((d.n_mu + AS_ROWS - 1) / AS_ROWS, n_img);
         dc::ProfScope ps(dc::KID_ADJ_S, st);
-        k_adj_from_s<<<grid, 256, sizeof(float) * AS_ROWS * g->NSp, st>>>(la, S);
+        if (quad) {
+          dim3 grid((d.n_mu + AS4_ROWS - 1) / AS4_ROWS, (n_img + 3) / 4);
+          DC_CUDA(cudaFuncSetAttribute(k_adj_from_s4, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       AS4_ROWS * 2048 * 16));
+          k_adj_from_s4<<<grid, 256, sizeof(float4) * AS4_ROWS * g->NSp, st>>>(la, S);
+        } else {
+          dim3 grid((d.n_mu + AS_ROWS - 1) / AS_ROWS, n_img);
+          k_adj_from_s<<<grid, 256, sizeof(float) * AS_ROWS * g->NSp, st>>>(la, S);
+        }
         DC_CHECK_LAUNCH("k_adj_from_s");
       }
       if (grad_W) {
         size_t total = (size_t)nv * d.n_mu * d.n_s;
         int nb = (int)std::min<size_t>((total + 255) / 256, 4096);
         dc::ProfScope ps(dc::KID_REDUCE_W, st);
-        k_reduce_gradW<<<nb, 256, 0, st>>>(g->w_sinoA, d.n_mu, d.n_s, g->NSp, bc, v0, nv,
-                                           b0 > 0, grad_W);
+        auto reduce = quad ? k_reduce_gradW<true> : k_reduce_gradW<false>;
+        reduce<<<nb, 256, 0, st>>>(g->w_sinoA, d.n_mu, d.n_s, g->NSp, bc, v0, nv, b0 > 0, grad_W);
         DC_CHECK_LAUNCH("k_reduce_gradW");
       }
       if (grad_g) {
@@ -1605,7 +1656,7 @@ int dc_filter_adjoint_from_s(const dc_geometry *g, int B, const float *grad_gF,
         ba.weight = WT_COS;
         ba.out_kind = OUT_F32;
         ba.out = grad_g;
-        if ((rc = launch_bp2d(g, ba, st))) return rc;
+        if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
       }
     }
   }
@@ -1663,20 +1714,26 @@ int dc_radon2d_adjoint(const dc_geometry *g, int B, const float *R, float *img, 
     return dc::fail(DC_ERR_UNSUPPORTED, "dc_radon2d_adjoint: ds < pitch/3 is not supported");
   cudaStream_t st = (cudaStream_t)stream;
   Chunking ck = chunking(g, B);
+  const bool quad = use_quad(g, ck.bc, ck.cv);
   for (int b0 = 0; b0 < B; b0 += ck.bc) {
     int bc = std::min(ck.bc, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += ck.cv) {
       int n_img = std::min(ck.cv, d.n_views - v0) * bc;
-      dim3 grid(64, n_img);
-      dc::ProfScope ps(dc::KID_SINO_IN, st);
-      k_sino_in<<<grid, 256, 0, st>>>(R, g->mu, d.n_mu, d.n_s, g->NSp, d.n_views, bc, v0, b0,
-                                      g->w_sinoA);
-      DC_CHECK_LAUNCH("k_sino_in");
+      {
+        dc::ProfScope ps(dc::KID_SINO_IN, st);
+        if (quad)
+          k_sino_in4<<<dim3(64, (n_img + 3) / 4), 256, 0, st>>>(
+              R, g->mu, d.n_mu, d.n_s, g->NSp, d.n_views, bc, v0, b0, n_img, (float4 *)g->w_sinoA);
+        else
+          k_sino_in<<<dim3(64, n_img), 256, 0, st>>>(R, g->mu, d.n_mu, d.n_s, g->NSp, d.n_views,
+                                                     bc, v0, b0, g->w_sinoA);
+        DC_CHECK_LAUNCH("k_sino_in");
+      }
       BP2Args ba = bp2_args(g, bc, v0, b0, n_img, g->w_sinoA);
       ba.weight = WT_NONE;
       ba.out_kind = OUT_F32;
       ba.out = img;
-      if ((rc = launch_bp2d(g, ba, st))) return rc;
+      if ((rc = launch_bp2d(g, ba, quad, st))) return rc;
     }
   }
   return DC_OK;

@@ -1,5 +1,6 @@
-// dc_filter_quad.cuh -- the line sums of four detector images at once (part
-// of dc_filter.cu: uses its LineArgs and epilogue helpers).
+// dc_filter_quad.cuh -- the line sums and the 2-D backprojection of four
+// detector images at once (part of dc_filter.cu: uses its argument structs
+// and epilogue helpers).
 //
 // A Joseph line depends on the angle, the s-bin and the principal point
 // only, so images that share the principal point (the views of one scanner,
@@ -372,21 +373,17 @@ __global__ void __launch_bounds__(L4_THREADS, 1)
       }
       continue;
     }
+    float4 *sA = reinterpret_cast<float4 *>(a.sinoA) + ((size_t)grp * a.n_mu + m) * a.NSp + k;
     if (MODE == M_DIFFSTORE) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (i < nv) a.sinoA[((size_t)(4 * grp + i) * a.n_mu + m) * a.NSp + k] = e[i];
+      *sA = e4;
       continue;
     }
     const bool on = k <= a.n_s - 2;
-    float w[4], t[4], y[4];
+    float w[4], y[4], tW[4];
+    const float4 t4 = (MODE == M_ADJ) ? *sA : make_float4(0, 0, 0, 0);
+    const float t[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      w[i] = (on && a.Wred) ? a.Wred[(vm[i] + m) * a.n_s + k] : 0.5f;
-      t[i] = (MODE == M_ADJ && on && i < nv)
-                 ? a.sinoA[((size_t)(4 * grp + i) * a.n_mu + m) * a.NSp + k]
-                 : 0.0f;
-    }
+    for (int i = 0; i < 4; ++i) w[i] = (on && a.Wred) ? a.Wred[(vm[i] + m) * a.n_s + k] : 0.5f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const dc::FView &fv = fvs[i];
@@ -400,15 +397,15 @@ __global__ void __launch_bounds__(L4_THREADS, 1)
         if (a.Sout && i < nv && k < a.n_s)
           a.Sout[(bvm[i] + m) * a.n_s + k] = on ? e[i] * wsino / a.ds : 0.0f;
       } else {  // M_ADJ: as in linesum_body
-        float tW = 0.0f;
+        tW[i] = 0.0f;
         if (on) {
           const float Qg = -a.cT * t[i] / a.ds;  // D_b^T of dL/dP
-          tW = Kv * (wsino * e[i] / a.ds) * Qg;
+          tW[i] = Kv * (wsino * e[i] / a.ds) * Qg;
           y[i] = wsino * w[i] * Kv * Qg;
         }
-        if (i < nv) a.sinoA[((size_t)(4 * grp + i) * a.n_mu + m) * a.NSp + k] = tW;
       }
     }
+    if (MODE == M_ADJ) *sA = make_float4(tW[0], tW[1], tW[2], tW[3]);
     ep[idx] = make_float4(y[0], y[1], y[2], y[3]);
   }
   if (MODE == M_RAW || MODE == M_GRANGEAT || MODE == M_DIFFSTORE) return;
@@ -422,12 +419,327 @@ __global__ void __launch_bounds__(L4_THREADS, 1)
     const float js = lmu[ml].jscale;
     const float4 c4 = ep[idx], p4 = (k > 0) ? ep[idx - 1] : make_float4(0, 0, 0, 0);
     const float c[4] = {c4.x, c4.y, c4.z, c4.w}, p[4] = {p4.x, p4.y, p4.z, p4.w};
-    float *dst = (MODE == M_FILTER) ? a.out : a.sinoB;
+    float val[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      float val = (MODE == M_FILTER) ? (c[i] - p[i]) / a.ds * a.cT * js : (p[i] - c[i]) / a.ds * js;
-      if (k >= a.n_s) val = 0.0f;
-      if (i < nv) dst[((size_t)(4 * grp + i) * a.n_mu + m) * a.NSp + k] = val;
+      val[i] = (MODE == M_FILTER) ? (c[i] - p[i]) / a.ds * a.cT * js : (p[i] - c[i]) / a.ds * js;
+      if (k >= a.n_s) val[i] = 0.0f;
+    }
+    reinterpret_cast<float4 *>(MODE == M_FILTER ? a.out : a.sinoB)[((size_t)grp * a.n_mu + m) *
+                                                                       a.NSp + k] =
+        make_float4(val[0], val[1], val[2], val[3]);
+  }
+}
+
+// the last step of the filter's reverse mode from a kept S (k_adj_from_s) on
+// quad sinograms: a CTA takes AS_ROWS angles of four images
+constexpr int AS4_ROWS = 2;
+__global__ void __launch_bounds__(256) k_adj_from_s4(LineArgs a, const float *__restrict__ S) {
+  extern __shared__ __align__(16) float4 ys4[];  // [AS4_ROWS][NSp]
+  const int grp = blockIdx.y, m0 = blockIdx.x * AS4_ROWS;
+  const int total = min(AS4_ROWS, a.n_mu - m0) * a.NSp;
+  float4 *sA = reinterpret_cast<float4 *>(a.sinoA) + ((size_t)grp * a.n_mu + m0) * a.NSp;
+  float4 *sB = reinterpret_cast<float4 *>(a.sinoB) + ((size_t)grp * a.n_mu + m0) * a.NSp;
+  bool bad_w = false;
+  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    const int m = m0 + idx / a.NSp, k = idx % a.NSp;
+    const bool on = k <= a.n_s - 2;
+    const float4 t4 = sA[idx];
+    const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+    const float sh = s_half_of(k, a.n_s, a.ds);
+    float y[4], tW[4], w[4], Sv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int n = min(4 * grp + i, a.n_img - 1), v = a.v0 + n / a.B, b = a.b0 + n % a.B;
+      w[i] = (on && a.Wred) ? a.Wred[((size_t)v * a.n_mu + m) * a.n_s + k] : 0.5f;
+      Sv[i] = on ? S[(((size_t)b * a.V + v) * a.n_mu + m) * a.n_s + k] : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int n = min(4 * grp + i, a.n_img - 1);
+      const dc::FView fv = a.fv[a.v0 + n / a.B];
+      const float D2 = fv.D * fv.D;
+      y[i] = tW[i] = 0.0f;
+      if (on) {
+        const float wsino = fmaf(sh, sh, D2) / D2;
+        const float Qg = -a.cT * t[i] / a.ds;  // D_b^T of dL/dP
+        const float Kv = redundancy_k(a.mu[m], fv, sh);
+        bad_w |= !isfinite(w[i]);
+        tW[i] = Kv * Sv[i] * Qg;
+        y[i] = wsino * w[i] * Kv * Qg;
+      }
+    }
+    sA[idx] = make_float4(tW[0], tW[1], tW[2], tW[3]);
+    ys4[idx] = make_float4(y[0], y[1], y[2], y[3]);
+  }
+  if (bad_w) atomicOr(a.err, DC_FLAG_NONFINITE_W);
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    const int k = idx % a.NSp;
+    float4 val = make_float4(0, 0, 0, 0);
+    if (k < a.n_s) {
+      const float js = a.mu[m0 + idx / a.NSp].jscale;
+      const float4 ym = (k > 0) ? ys4[idx - 1] : make_float4(0, 0, 0, 0);
+      const float4 y0 = ys4[idx];  // 0 at k = n_s - 1
+      val = make_float4((ym.x - y0.x) / a.ds * js, (ym.y - y0.y) / a.ds * js,
+                        (ym.z - y0.z) / a.ds * js, (ym.w - y0.w) / a.ds * js);
+    }
+    sB[idx] = val;
+  }
+}
+
+// k_sino_in for four images: user sinograms into quads, times the Joseph scale
+__global__ void k_sino_in4(const float *__restrict__ R, const dc::MuRec *__restrict__ mu, int n_mu,
+                           int n_s, int NSp, int V, int B, int v0, int b0, int n_img,
+                           float4 *__restrict__ dst) {
+  const int grp = blockIdx.y;
+  const size_t total = (size_t)n_mu * NSp;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+       i += (size_t)gridDim.x * blockDim.x) {
+    const int m = (int)(i / NSp), k = (int)(i % NSp);
+    float val[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = 4 * grp + q, v = v0 + n / B, b = b0 + n % B;
+      val[q] = (k < n_s && n < n_img) ? R[(((size_t)b * V + v) * n_mu + m) * n_s + k] * mu[m].jscale
+                                      : 0.0f;
+    }
+    dst[(size_t)grp * total + i] = make_float4(val[0], val[1], val[2], val[3]);
+  }
+}
+
+// -------------------------------------------- 2-D backprojection, four images
+// As for the line sums: position, floor, hat weights and address of a
+// (pixel, angle) pair once for four images, their taps one 16-byte load each.
+// The bare pair then runs at 15.8 pairs per clock and SM (128 B / 8 B = 16 at
+// most); the per-image kernel reaches 9.3, bound by instructions.
+//
+// A CTA takes a tile of 2048 (or, for grids too small to fill the GPU, 512)
+// pixels: 8 warps of 32 columns x RY rows, nwx warps side by side.  Only the
+// s-window that a tile meets is staged, per angle: TMA boxes of the quad
+// sinogram, zeros outside [0, NSp), so no position is clamped.  A thread holds
+// RY pixels x 4 images.
+constexpr int B4_THREADS = 256;
+constexpr int B4_MC = 16;  // angles per stage
+struct B4Shape {
+  int nwx;       // warps side by side
+  int lwb, nb;   // boxes of lwb bins (multiple of 8, at most 64), nb of them per angle
+};
+
+struct B4Mu {
+  float F00, Bc, Bs, winv;
+  float w1c;
+  unsigned cbase;  // byte offset of bin I00 in its stage row, minus the floor's exponent bits
+  unsigned pad0, pad1;
+};
+
+// taps per pixel and angle: the hat's half-width is at most pitch / ds bins
+template <int NT>
+constexpr int b4_left() { return NT / 2 - 1; }
+
+inline int b4_taps(double pitch, double ds) {
+  return ds >= pitch * (1.0 - 1e-12) ? 2 : 2.0 * ds >= pitch * (1.0 - 1e-12) ? 4 : 6;
+}
+
+// the warps' arrangement with the fewest pixels outside the detector (the
+// squarest of equals: the smallest window), and the window of its tile
+inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY) {
+  B4Shape s;
+  long best = 0;
+  const int order[4] = {2, 1, 4, 8};
+  for (int i = 0; i < 4; ++i) {
+    const int tx = 32 * order[i], ty = RY * (8 / order[i]);
+    const long px = (long)((W + tx - 1) / tx) * tx * ((H + ty - 1) / ty) * ty;
+    if (i == 0 || px < best) {
+      best = px;
+      s.nwx = order[i];
+    }
+  }
+  const int tx = 32 * s.nwx, ty = RY * (8 / s.nwx), nt = b4_taps(pitch, ds);
+  const double span = std::sqrt((tx - 1.0) * (tx - 1.0) + (ty - 1.0) * (ty - 1.0)) * pitch / ds;
+  const int need = (int)(span + 0.1) + 3 + nt;
+  s.nb = (need + 63) / 64;
+  s.lwb = (((need + s.nb - 1) / s.nb) + 7) & ~7;
+  return s;
+}
+
+// Rows per thread: 8, unless the 2048-pixel tiles of the views at hand leave
+// SMs without a CTA, then 2 (64 views of 64 x 64, 32 tiles: 35 us against 70;
+// 90 views of 128 x 128, 184 tiles: 168 against 158).  A property of the
+// geometry, so that an image's result does not depend on the chunk or batch
+// that it comes in.
+inline int b4_rows(int H, int W, double pitch, double ds, int images) {
+  const B4Shape s = b4_shape(H, W, pitch, ds, 8);
+  const int tx = 32 * s.nwx, ty = 64 / s.nwx;
+  const long tiles = (long)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * ((images + 3) / 4);
+  return tiles < 152 ? 2 : 8;
+}
+
+// 8 rows per thread want the registers of two CTAs per SM (496 images of 384 x
+// 512 and 720 angles: 22.1 ms with the per-image kernel, 16.2 with three CTAs
+// at 80 registers, waiting for shared memory; 15.1 with two: 14.8 pairs per
+// clock and SM)
+template <int NT, int RY>
+__global__ void __launch_bounds__(B4_THREADS, RY == 8 ? 2 : 4)
+    k_bp2d4(BP2Args a, B4Shape sh, const __grid_constant__ CUtensorMap tm) {
+  extern __shared__ __align__(1024) unsigned char dyn[];
+  __shared__ uint64_t full[2];
+  __shared__ __align__(16) B4Mu bmu[2][B4_MC];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = blockIdx.z;
+  const int tx = 32 * sh.nwx, ty = RY * (8 / sh.nwx);
+  const int j0 = blockIdx.x * tx, r0 = blockIdx.y * ty;
+  const int row_bytes = sh.lwb * sh.nb * 16;
+  const int nchunk = (a.n_mu + B4_MC - 1) / B4_MC;
+  constexpr int TL = b4_left<NT>();
+
+  // constants of chunk c's angles for this tile (exact float splits of the
+  // origin, as in the per-image kernel) and the copies of their s-windows:
+  // one thread per angle
+  auto stage = [&](int c) {
+    const int st = c & 1, nm = min(B4_MC, a.n_mu - c * B4_MC);
+    dc::fence_proxy_async();
+    if (tid == 0) dc::mbar_arrive_expect_tx(&full[st], (unsigned)(nm * row_bytes));
+    __syncwarp();
+    if (tid < nm) {
+      const int m = c * B4_MC + tid;
+      const dc::MuRec R = a.mu[m];
+      const dc::VMu Q = a.vmu[m];  // the principal point is the same for every view
+      const float fj0 = (float)j0, fr0 = (float)r0;
+      const float t = fj0 * R.bc_hi + fr0 * R.bs_hi;  // exact
+      const float ti = floorf(t);
+      const float F = Q.xof + (t - ti) + fmaf(fj0, R.bc_lo, fr0 * R.bs_lo);
+      const float Fi = floorf(F);
+      const int I00 = (int)(Q.xoi + ti + Fi);
+      B4Mu M;
+      M.F00 = F - Fi;
+      M.Bc = R.bc_hi + R.bc_lo;
+      M.Bs = R.bs_hi + R.bs_lo;
+      M.winv = R.winv;
+      M.w1c = 1.0f - R.winv;
+      const float ex = (float)(tx - 1) * M.Bc, ey = (float)(ty - 1) * M.Bs;
+      // first bin of the window relative to I00, with a margin for the
+      // rounding of the positions
+      const int kw = (int)floorf(M.F00 + fminf(ex, 0.0f) + fminf(ey, 0.0f) - 0.01f) - TL;
+      M.cbase = (unsigned)(st * B4_MC * row_bytes + tid * row_bytes - kw * 16) - 16u * 0x4B400000u;
+      M.pad0 = M.pad1 = 0u;
+      bmu[st][tid] = M;
+      unsigned char *dst = dyn + (size_t)(st * B4_MC + tid) * row_bytes;
+      for (int q = 0; q < sh.nb; ++q)
+        dc::tma_load_3d(dst + q * sh.lwb * 16, &tm, (I00 + kw + q * sh.lwb) * 4, m, grp, &full[st]);
+    }
+  };
+  if (tid == 0) {
+    dc::mbar_init(&full[0], 1);
+    dc::mbar_init(&full[1], 1);
+    dc::fence_barrier_init();
+  }
+  __syncthreads();
+  if (warp == 0) {
+    stage(0);
+    if (nchunk > 1) stage(1);
+  }
+  __syncthreads();
+
+  float2 acc[RY][2];
+#pragma unroll
+  for (int r = 0; r < RY; ++r) acc[r][0] = acc[r][1] = make_float2(0.0f, 0.0f);
+  const int jl = (warp & (sh.nwx - 1)) * 32 + lane, rl = (warp / sh.nwx) * RY;
+  const float jlf = (float)jl;
+  float2 rlf[RY / 2];  // tile rows of the thread's pixels in pairs
+#pragma unroll
+  for (int r = 0; r < RY / 2; ++r) rlf[r] = make_float2((float)(rl + 2 * r), (float)(rl + 2 * r + 1));
+  const float2 M2 = make_float2(12582912.0f, 12582912.0f);
+  const float2 mM2 = make_float2(-12582912.0f, -12582912.0f), m12 = make_float2(-1.0f, -1.0f);
+  const unsigned sbase = dc::smem_addr(dyn);
+
+  bool ok = true;
+  int c = 0;
+  for (; c < nchunk; ++c) {
+    if (!dc::mbar_wait_bounded(&full[c & 1], (c >> 1) & 1, a.err)) ok = false;
+    const int nm = min(B4_MC, a.n_mu - c * B4_MC);
+    for (int mi = 0; mi < nm; ++mi) {
+      const B4Mu M = bmu[c & 1][mi];
+      const unsigned cb = M.cbase + sbase;
+      const float base = fmaf(jlf, M.Bc, M.F00);
+      const float2 base2 = make_float2(base, base), Bs2 = make_float2(M.Bs, M.Bs);
+#pragma unroll
+      for (int r = 0; r < RY / 2; ++r) {
+        const float2 x = __ffma2_rn(rlf[r], Bs2, base2);
+        const float2 t = __fadd2_rd(x, M2);  // exact floor and fraction
+        const float2 f = __ffma2_rn(__fadd2_rn(t, mM2), m12, x);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float fh = h ? f.y : f.x;
+          const unsigned ad = __float_as_uint(h ? t.y : t.x) * 16u + cb;
+          float2 &a0 = acc[2 * r + h][0], &a1 = acc[2 * r + h][1];
+#pragma unroll
+          for (int q = 0; q < NT; ++q) {
+            // tap floor(x) + q - TL at distance |f + TL - q|: for ds >= pitch
+            // (winv >= 1) the hat never exceeds 1 and the clamp at 0 is a
+            // saturation
+            float w;
+            if (NT == 2)
+              w = __saturatef(q == 0 ? fmaf(-fh, M.winv, 1.0f) : fmaf(fh, M.winv, M.w1c));
+            else
+              w = fmaxf(0.0f, fmaf(-fabsf(fh + (float)(TL - q)), M.winv, 1.0f));
+            const float2 w2 = make_float2(w, w);
+            const float4 p = lds128(ad + (unsigned)(16 * (q - TL)));
+            a0 = __ffma2_rn(w2, make_float2(p.x, p.y), a0);
+            a1 = __ffma2_rn(w2, make_float2(p.z, p.w), a1);
+          }
+        }
+      }
+    }
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      break;
+    }
+    if (warp == 0 && c + 2 < nchunk) stage(c + 2);
+  }
+  if (!ok) {  // a copy never landed: nothing may be in flight when the CTA ends
+    dc::mbar_wait_bounded(&full[c & 1], (c >> 1) & 1, nullptr);
+    if (c + 1 < nchunk) dc::mbar_wait_bounded(&full[(c + 1) & 1], ((c + 1) >> 1) & 1, nullptr);
+    return;
+  }
+
+  const int j = j0 + jl;
+  float lmax[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (j < a.W) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int n = 4 * grp + i;
+      if (n >= a.n_img) break;
+      const int v = a.v0 + n / a.B, b = a.b0 + n % a.B;
+      const dc::FView fv = a.fv[v];
+      const float xx = (j - fv.cu) * a.pitch;
+#pragma unroll
+      for (int r = 0; r < RY; ++r) {
+        const int rr = r0 + rl + r;
+        if (rr >= a.H) break;
+        float val = (i & 1) ? acc[r][i >> 1].y : acc[r][i >> 1].x;
+        if (a.weight != WT_NONE) {
+          const float yy = (rr - fv.cv) * a.pitch;
+          const float l2 = fmaf(xx, xx, fmaf(yy, yy, fv.D * fv.D));
+          val *= (a.weight == WT_D) ? l2 : fv.D * rsqrtf(l2);
+        }
+        if (a.out_kind == OUT_F32_ABSMAX || a.out_kind == OUT_F32_SLOT) {
+          ((float *)a.out)[((size_t)n * a.H + rr) * a.Wp + j] = val;
+          lmax[i] = fmaxf(lmax[i], fabsf(val));
+        } else {
+          const size_t o = (((size_t)b * a.V + v) * a.H + rr) * a.W + j;
+          if (a.out_kind == OUT_BF16) ((__nv_bfloat16 *)a.out)[o] = __float2bfloat16_rn(val);
+          else ((float *)a.out)[o] = val;
+        }
+      }
+    }
+  }
+  if (a.out_kind == OUT_F32_ABSMAX) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float l = lmax[i];
+      for (int o = 16; o > 0; o >>= 1) l = fmaxf(l, __shfl_xor_sync(0xffffffffu, l, o));
+      if (lane == 0 && 4 * grp + i < a.n_img) atomicMax(&a.absmax[4 * grp + i], __float_as_uint(l));
     }
   }
 }
