@@ -92,3 +92,22 @@ def test_compare_reports_learned_and_analytic_weights():
     for k in ("learned", "half", "eq9"):
         assert np.isfinite(res["test_rel_mse"][k])
     assert res["loss_last_epoch"] < res["loss_first_epoch"]
+
+
+# lines at the edges of the tiles (128 outputs, 64 lines), one and two samples,
+# a halo longer than the line, no halo, the largest radius of the tiled kernel
+# and the first beyond it
+@pytest.mark.parametrize("V,n_mu,n_s,sigma,radius", [(1, 127, 65, 20.0, 60), (2, 128, 66, 7.0, 16),
+                                                     (1, 129, 130, 20.0, 60), (1, 257, 64, 4.0, 1),
+                                                     (3, 1, 129, 5.0, 20), (1, 2, 3, 5.0, 40),
+                                                     (1, 33, 40, 1.0, 0), (1, 150, 70, 90.0, 320),
+                                                     (1, 150, 70, 90.0, 321)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_gauss_smooth_tile_edges(V, n_mu, n_s, sigma, radius, adjoint):
+    rng = np.random.default_rng(n_mu * 7 + n_s)
+    W = rng.normal(size=(V, n_mu, n_s)).astype(np.float32)
+    got = api.dc_gauss_smooth(torch.as_tensor(W, device="cuda"), sigma, radius, adjoint=adjoint)
+    ref = orc.gauss_smooth(W, sigma, radius, adjoint=adjoint)
+    got = got.double().cpu().numpy()
+    assert rel_l2(got[..., :-1], ref[..., :-1]) < 1e-5
+    np.testing.assert_array_equal(got[..., -1], W[..., -1])
