@@ -201,10 +201,18 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
 int backproject_check(const dc_geometry *g, int B, const void *gF, int dtype,
                       const float *gF_scale, const float *vol, unsigned flags, const char *who);
 // backprojection of the z range [z_begin, z_end) of every batch item with the
-// TMA kernel; *used = false (nothing launched) when that kernel cannot run
+// staged kernels; *used = false (nothing launched) when they cannot run
 int backproject_slab(const dc_geometry *g, int B, const void *gF, int dtype,
                      const float *gF_scale, float *vol, unsigned flags, int z_begin, int z_end,
                      cudaStream_t st, bool *used);
+// the same with footprints staged by rows (dc_backproject_rows.cu), for g^F
+// whose rows TMA cannot address; *used = false when the pairs of DC_F32X2 are
+// not 8-byte aligned
+int backproject_rows(const dc_geometry *g, int B, const void *gF, int dtype,
+                     const float *gF_scale, float *vol, unsigned flags, int z_begin, int z_end,
+                     cudaStream_t st, bool *used);
+// the backprojection's box depth for this geometry (g->bp_nz)
+void bp_plan(dc_geometry *g);
 // the batched persistent filter (dc_filter.cu): one launch filters every
 // view of up to 32 problems into the given g^F buffers (and FP16 scales)
 struct BatchFilterPlan;

@@ -1288,7 +1288,7 @@ int alloc_workspace(dc_geometry *g) {
   if (g->quad) ci &= ~3;
   g->chunk_images = ci;
   g->chunk_capacity = ci;
-  g->bp_nz = 32;
+  bp_plan(g);
   g->ls_rb = linesum_band_rows(d.det_rows, d.det_cols, g->mg, g->NSp);
   if (g->ls_rb == 0 || bp2d_smem(g) > 200 * 1024)
     return fail(DC_ERR_UNSUPPORTED, "detector or sinogram rows too long for shared memory");
