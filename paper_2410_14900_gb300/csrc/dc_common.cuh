@@ -149,6 +149,7 @@ struct dc_geometry {
   // work area
   int chunk_images;          // images (view x batch item) per chunk
   int chunk_capacity;        // images the work area was sized for
+  int l2_images;             // images whose per-image work area stays in L2
   int bp_nz;                 // voxels per thread along z in the backprojector (16, 32)
   size_t img_stride;         // floats per padded image  (H * Wp)
   size_t sino_stride;        // floats per padded sinogram (n_mu * NSp)
@@ -190,8 +191,8 @@ int quad_plan(dc_geometry *g);
 // argument checks of the filter entry points (DC_OK or the error code)
 int filter_check(const dc_geometry *g, int B, const float *gin, const void *gF, int dtype,
                  const float *gF_scale, const char *who);
-// chunk sizes: bc batch items of cv views per chunk of the work area
-void filter_chunk_plan(const dc_geometry *g, int B, int *bc, int *cv);
+// chunk sizes for a storage form: bc batch items of cv views per chunk of the work area
+void filter_chunk_plan(const dc_geometry *g, int B, int dtype, int *bc, int *cv);
 // the filter of one chunk: views [v0, v0 + nv) of items [b0, b0 + bc)
 // (S: optional [B][V][n_mu][n_s] copy of Grangeat's function, or NULL)
 int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *gF, int dtype,

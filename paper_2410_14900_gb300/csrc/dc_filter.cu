@@ -1087,6 +1087,14 @@ Chunking chunking(const dc_geometry *g, int B, int view_limit = 0) {
 // chunk, so that every image of a call takes the same path.
 bool use_quad(const dc_geometry *g, int bc, int cv) { return g->quad && bc * cv >= 2; }
 
+// BF16 storage keeps the per-image kernels.  The two paths' FP32 results
+// differ by their rounding (5e-6 relative), which turns 0.1 % of the BF16
+// roundings the other way, each by 2^-8 of its value; the reconstructions that
+// differ by that (2.2e-5 relative, 1.5e-3 at most) are further apart than FP32
+// results of one input may be from release to release (2e-5, 8e-4).  FP16's
+// roundings, eight times finer, stay inside (5e-6, 6e-5).
+bool quad_storage(int dtype) { return dtype != DC_BF16; }
+
 // ------------------------------------------------ batched persistent filter
 // One kernel filters every view of a batch of problems (orbits with uneven
 // view counts, detectors and angle grids): persistent CTAs of BF_THREADS
@@ -1286,6 +1294,8 @@ int alloc_workspace(dc_geometry *g) {
   if (ci < 4) ci = 4;
   if (ci > 256) ci = 256;
   if (g->quad) ci &= ~3;
+  g->l2_images = std::max(4, (int)((112L << 20) /
+                                   (long)((g->img_stride + 2 * g->sino_stride) * sizeof(float))));
   g->chunk_images = ci;
   g->chunk_capacity = ci;
   bp_plan(g);
@@ -1334,8 +1344,13 @@ int filter_check(const dc_geometry *g, int B, const float *gin, const void *gF, 
   return DC_OK;
 }
 
-void filter_chunk_plan(const dc_geometry *g, int B, int *bc, int *cv) {
+void filter_chunk_plan(const dc_geometry *g, int B, int dtype, int *bc, int *cv) {
+  // the per-image kernels take chunks that stay in L2
   Chunking ck = chunking(g, B);
+  if (g->quad && !quad_storage(dtype)) {
+    ck.bc = std::min(ck.bc, g->l2_images);
+    ck.cv = std::max(1, std::min(ck.cv, g->l2_images / ck.bc));
+  }
   *bc = ck.bc;
   *cv = ck.cv;
 }
@@ -1346,7 +1361,7 @@ int filter_chunk(const dc_geometry *g, const float *gin, const float *W, void *g
   const dc_geometry_desc &d = g->d;
   const int n_img = nv * bc;
   int rc;
-  const bool quad = use_quad(g, g->chunk_images, 1);
+  const bool quad = use_quad(g, g->chunk_images, 1) && quad_storage(dtype);
   if ((rc = launch_prep(g, gin, WT_COS, v0, n_img, bc, b0, quad, st))) return rc;
   LineArgs la = line_args(g, bc, v0, b0, n_img);
   la.Wred = W;
@@ -1531,7 +1546,7 @@ static int filter_all(const dc_geometry *g, int B, const float *gin, const float
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   int bcm, cvm;
-  dc::filter_chunk_plan(g, B, &bcm, &cvm);
+  dc::filter_chunk_plan(g, B, dtype, &bcm, &cvm);
   for (int b0 = 0; b0 < B; b0 += bcm) {
     int bc = std::min(bcm, B - b0);
     for (int v0 = 0; v0 < g->d.n_views; v0 += cvm) {

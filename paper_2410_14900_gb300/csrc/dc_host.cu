@@ -55,7 +55,7 @@ extern "C" int dc_reconstruct_host(const dc_geometry *geom, int B, const float *
   // filter, chunk by chunk behind the uploads
   const size_t img = (size_t)d.det_rows * d.det_cols;
   int bcm, cvm, k = 0;
-  dc::filter_chunk_plan(g, B, &bcm, &cvm);
+  dc::filter_chunk_plan(g, B, dtype, &bcm, &cvm);
   for (int b0 = 0; b0 < B; b0 += bcm) {
     const int bc = std::min(bcm, B - b0);
     for (int v0 = 0; v0 < d.n_views; v0 += cvm) {
