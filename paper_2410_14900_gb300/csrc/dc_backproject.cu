@@ -100,85 +100,6 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_bp3d(BPArgs a) {
   }
 }
 
-struct BPAdjArgs {
-  const float *grad_vol;
-  const float *relu_vol;
-  const dc::BPView *views;
-  float *grad_gF;
-  int V, H, W, nx, ny, nz, B;
-  float dx, dy, dz;
-};
-
-// transpose: every voxel scatters its weighted gradient onto the four taps
-__global__ void __launch_bounds__(BP_TX *BP_TY) k_bp3d_adj(BPAdjArgs a) {
-  __shared__ dc::BPView sv[BP_VCHUNK];
-  const int ix = blockIdx.x * BP_TX + threadIdx.x;
-  const int iy = blockIdx.y * BP_TY + threadIdx.y;
-  const int zblocks = (a.nz + BP_NZ - 1) / BP_NZ;
-  const int b = blockIdx.z / zblocks;
-  const int z0 = (blockIdx.z % zblocks) * BP_NZ;
-  const int tid = threadIdx.y * BP_TX + threadIdx.x;
-  const float xo = ((float)ix - 0.5f * (float)(a.nx - 1)) * a.dx;
-  const float yo = ((float)iy - 0.5f * (float)(a.ny - 1)) * a.dy;
-  const float zo = ((float)z0 - 0.5f * (float)(a.nz - 1)) * a.dz;
-  const size_t np = (size_t)a.H * a.W;
-  const size_t nvox = (size_t)a.nx * a.ny * a.nz;
-  const bool inside = (ix < a.nx && iy < a.ny);
-  float gv[BP_NZ];
-#pragma unroll
-  for (int k = 0; k < BP_NZ; ++k) {
-    int iz = z0 + k;
-    gv[k] = 0.0f;
-    if (inside && iz < a.nz) {
-      size_t o = (size_t)b * nvox + ((size_t)iz * a.ny + iy) * a.nx + ix;
-      float g = a.grad_vol[o];
-      if (a.relu_vol && !(a.relu_vol[o] > 0.0f)) g = 0.0f;
-      gv[k] = g;
-    }
-  }
-  float *gbase = a.grad_gF + (size_t)b * a.V * np;
-  for (int i0 = 0; i0 < a.V; i0 += BP_VCHUNK) {
-    int nvc = min(BP_VCHUNK, a.V - i0);
-    __syncthreads();
-    if (tid < nvc) sv[tid] = a.views[i0 + tid];
-    __syncthreads();
-    if (!inside) continue;
-    for (int ii = 0; ii < nvc; ++ii) {
-      const dc::BPView w = sv[ii];
-      float *img = gbase + (size_t)(i0 + ii) * np;
-      float U0 = fmaf(w.r0.x, xo, fmaf(w.r0.y, yo, fmaf(w.r0.z, zo, w.r0.w)));
-      float V0 = fmaf(w.r1.x, xo, fmaf(w.r1.y, yo, fmaf(w.r1.z, zo, w.r1.w)));
-      float W0 = fmaf(w.r2.x, xo, fmaf(w.r2.y, yo, fmaf(w.r2.z, zo, w.r2.w)));
-      float dU = w.r0.z * a.dz, dV = w.r1.z * a.dz, dW = w.r2.z * a.dz;
-      float ex = w.ca.x + xo, ey = w.ca.y + yo, ez0 = w.ca.z + zo;
-      float rho2 = fmaf(ex, ex, ey * ey);
-#pragma unroll
-      for (int k = 0; k < BP_NZ; ++k) {
-        if (gv[k] == 0.0f) continue;
-        float kf = (float)k;
-        float dep = fmaf(kf, dW, W0);
-        if (!(dep > 0.0f)) continue;
-        float rw = __frcp_rn(dep);
-        float u = fmaf(fmaf(kf, dU, U0), rw, w.pp.x);
-        float v = fmaf(fmaf(kf, dV, V0), rw, w.pp.y);
-        float ez = fmaf(kf, a.dz, ez0);
-        float g = gv[k] * __frcp_rn(fmaf(ez, ez, rho2));
-        u = fminf(fmaxf(u, -2.0f), (float)a.W + 1.0f);
-        v = fminf(fmaxf(v, -2.0f), (float)a.H + 1.0f);
-        float fu, fv;
-        int j = dc::floor_frac(u, fu), r = dc::floor_frac(v, fv);
-        bool j0 = (j >= 0 && j < a.W), j1 = (j + 1 >= 0 && j + 1 < a.W);
-        bool r0 = (r >= 0 && r < a.H), r1 = (r + 1 >= 0 && r + 1 < a.H);
-        float *p = img + (ptrdiff_t)r * a.W + j;
-        if (r0 && j0) atomicAdd(p, g * (1.0f - fu) * (1.0f - fv));
-        if (r0 && j1) atomicAdd(p + 1, g * fu * (1.0f - fv));
-        if (r1 && j0) atomicAdd(p + a.W, g * (1.0f - fu) * fv);
-        if (r1 && j1) atomicAdd(p + a.W + 1, g * fu * fv);
-      }
-    }
-  }
-}
-
 template <typename T, bool KAHAN, int NZ>
 __global__ void __launch_bounds__(TB_TX *TB_TY, 2) k_bp3d_tma(BPArgs a, unsigned *err,
                                                              const __grid_constant__ CUtensorMap tmn,
@@ -258,270 +179,6 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 2) k_bp3d_batched(const BatchPro
       return;
     }
   }
-}
-
-// ------------------------------------------------------------------------
-// Transpose of the staged backprojection.  Same CTA boxes and footprints as
-// the forward kernel; for every view the CTA's voxels scatter their weighted
-// gradients into a shared-memory footprint tile (row stride 69: 5 mod 32, so
-// the rows a warp's lanes reach fall on different banks for most view
-// directions), which is then added to g^F's gradient with one global atomic
-// per non-zero pixel.  Two tiles alternate: a view's tile is flushed while
-// the next view scatters into the other, one barrier per view.
-//
-// The tile accumulates in 32-bit fixed point, because integer shared-memory
-// atomics are native while floating-point ones are not.  The unit is chosen
-// per (box, view) from a rigorous bound on any pixel sum: every voxel's four
-// bilinear weights sum to one, so a pixel gets at most the box's total,
-// nvox * max|g| / d_min^2, with d_min the source's distance to the box
-// (centre distance minus half-diagonal); tighter and still rigorous is
-// sum_box |g| / d_min^2, since every voxel's weights sum to one and each
-// voxel's distance is at least d_min.  That bound maps to 2^30, so the sums
-// cannot overflow; each contribution is rounded to the nearest unit.
-constexpr int TA_S = 69;
-static_assert(TA_S >= TB_BWW, "a tile row holds the widest footprint");
-static_assert(TB_NZ == 32, "the adjoint rotates each lane's voxel order by its lane index");
-static_assert(TB_BWW <= 64 && TB_BH <= 255, "the tile flush takes 32 columns per lane pass");
-
-__global__ void __launch_bounds__(TB_TX *TB_TY, 2) k_bp3d_adj_tile(BPAdjArgs a) {
-  __shared__ int tiles[2][TB_BH * TA_S];
-  __shared__ dc::BPView sv[TB_VCH];
-  __shared__ int4 vtab[TB_VCH];
-  __shared__ float wsum[TB_TX * TB_TY / 32];
-  __shared__ float wmax[TB_TX * TB_TY / 32];
-  const int tid = threadIdx.y * TB_TX + threadIdx.x;
-  const int ix = blockIdx.x * TB_TX + threadIdx.x;
-  const int iy = blockIdx.y * TB_TY + threadIdx.y;
-  const int zblocks = (a.nz + TB_NZ - 1) / TB_NZ;
-  const int b = blockIdx.z / zblocks;
-  const int z0 = (blockIdx.z % zblocks) * TB_NZ;
-  const float cx = 0.5f * (float)(a.nx - 1), cy = 0.5f * (float)(a.ny - 1),
-              cz = 0.5f * (float)(a.nz - 1);
-  const float xo = ((float)ix - cx) * a.dx;
-  const float yo = ((float)iy - cy) * a.dy;
-  const float zo = ((float)z0 - cz) * a.dz;
-  const float bx0 = ((float)(blockIdx.x * TB_TX) - cx) * a.dx;
-  const float bx1 = ((float)min(blockIdx.x * TB_TX + TB_TX - 1, a.nx - 1) - cx) * a.dx;
-  const float by0 = ((float)(blockIdx.y * TB_TY) - cy) * a.dy;
-  const float by1 = ((float)min(blockIdx.y * TB_TY + TB_TY - 1, a.ny - 1) - cy) * a.dy;
-  const float bz0 = zo;
-  const float bz1 = ((float)min(z0 + TB_NZ - 1, a.nz - 1) - cz) * a.dz;
-  // box centre and half-diagonal (for the distance bound)
-  const float bcx = 0.5f * (bx0 + bx1), bcy = 0.5f * (by0 + by1), bcz = 0.5f * (bz0 + bz1);
-  const float bhd = 0.5f * sqrtf((bx1 - bx0) * (bx1 - bx0) + (by1 - by0) * (by1 - by0) +
-                                 (bz1 - bz0) * (bz1 - bz0)) + 0.5f * (a.dx + a.dy + a.dz);
-  const size_t np = (size_t)a.H * a.W;
-  const size_t nvox = (size_t)a.nx * a.ny * a.nz;
-  const bool inside = (ix < a.nx && iy < a.ny);
-  // Lane l takes its column's voxels in the rotated order kz = (k + l) mod
-  // TB_NZ, so that at each step the lanes of a warp are at different depths
-  // along z: lanes whose columns project to the same detector column (the
-  // columns of a warp lined up with the view direction) then hit different
-  // detector rows, and the row stride of the tile (TA_S) spreads those rows
-  // over the banks.  The fixed-point sums are exact, so the order does not
-  // change the result.  gv[k] holds voxel kz.
-  const int rot = tid & 31;
-  const float rotf = (float)rot;
-  float gv[TB_NZ];
-  float gs = 0.0f, gm = 0.0f;
-#pragma unroll
-  for (int k = 0; k < TB_NZ; ++k) {
-    int iz = z0 + ((k + rot) & (TB_NZ - 1));
-    gv[k] = 0.0f;
-    if (inside && iz < a.nz) {
-      size_t o = (size_t)b * nvox + ((size_t)iz * a.ny + iy) * a.nx + ix;
-      float g = a.grad_vol[o];
-      if (a.relu_vol && !(a.relu_vol[o] > 0.0f)) g = 0.0f;
-      gv[k] = g;
-      gs += fabsf(g);
-      gm = fmaxf(gm, fabsf(g));
-    }
-  }
-  const bool any = gs > 0.0f;
-  for (int o = 16; o > 0; o >>= 1) {
-    gs += __shfl_xor_sync(0xffffffffu, gs, o);
-    gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
-  }
-  if ((tid & 31) == 0) {
-    wsum[tid >> 5] = gs;
-    wmax[tid >> 5] = gm;
-  }
-  for (int e = tid; e < 2 * TB_BH * TA_S; e += TB_TX * TB_TY) (&tiles[0][0])[e] = 0;
-  __syncthreads();
-  float gsum = 0.0f, gmax = 0.0f;
-  for (int q = 0; q < TB_TX * TB_TY / 32; ++q) {
-    gsum += wsum[q];
-    gmax = fmaxf(gmax, wmax[q]);
-  }
-  gsum *= 1.0001f;  // headroom for the rounding of this sum
-  if (!(gsum > 0.0f)) return;  // nothing to scatter from this box (CTA-uniform)
-  // One contribution is at most gmax / d^2 <= gmax / dmin^2, i.e. at most
-  // 2^30 gmax / gsum units.  When the box's gradient is spread over at least
-  // 512 voxels' worth of its largest value, every contribution stays below
-  // 2^21 units and is rounded to an integer by adding 1.5 * 2^23 (the sum
-  // has unit spacing, and round-to-nearest-even is the same rounding as
-  // __float2int_rn) instead of a conversion instruction.  CTA-uniform.
-  const bool magic_round = gsum >= 512.0f * gmax;
-  float *gbase = a.grad_gF + (size_t)b * a.V * np;
-
-  // The pending tile: the last scattered view's, flushed while the next view
-  // scatters into the other tile.  Its footprint rectangle (columns pt.w &
-  // 255, rows pt.w >> 8) holds every tap of the view (one pixel of margin on
-  // each side of the projected box), so flushing it clears the whole tile.
-  int cur = 0;
-  bool pending = false;
-  int4 pt = make_int4(0, 0, 0, 0);
-  float p_from_fix = 0.0f;
-  float *p_img = nullptr;
-  auto flush_pending = [&]() {
-    int *T = tiles[cur ^ 1];
-    const int nc = pt.w & 255, nr = pt.w >> 8;
-    for (int c = tid & 31; c < nc; c += 32) {
-      const int jj = pt.x + c;
-      for (int r = tid >> 5; r < nr; r += (TB_TX * TB_TY) >> 5) {
-        const int q = T[r * TA_S + c];
-        if (q != 0) {
-          T[r * TA_S + c] = 0;
-          const int rr = pt.y + r;
-          if (jj >= 0 && jj < a.W && rr >= 0 && rr < a.H)
-            atomicAdd(p_img + (size_t)rr * a.W + jj, (float)q * p_from_fix);
-        }
-      }
-    }
-  };
-
-  for (int c0 = 0; c0 < a.V; c0 += TB_VCH) {
-    const int nvc = min(TB_VCH, a.V - c0);
-    __syncthreads();
-    {  // footprints: thread = (view, corner), as in the forward kernel
-      const int vi = tid >> 3, cr = tid & 7;
-      float umin = 0.0f, umax = 0.0f, vmin = 0.0f, vmax = 0.0f;
-      int good = 1;
-      if (vi < nvc) {
-        const dc::BPView w = a.views[c0 + vi];
-        if (cr == 0) sv[vi] = w;
-        float X = (cr & 1) ? bx1 : bx0, Y = (cr & 2) ? by1 : by0, Z = (cr & 4) ? bz1 : bz0;
-        float U = fmaf(w.r0.x, X, fmaf(w.r0.y, Y, fmaf(w.r0.z, Z, w.r0.w)));
-        float Vv = fmaf(w.r1.x, X, fmaf(w.r1.y, Y, fmaf(w.r1.z, Z, w.r1.w)));
-        float Wd = fmaf(w.r2.x, X, fmaf(w.r2.y, Y, fmaf(w.r2.z, Z, w.r2.w)));
-        good = (Wd > 1.0f);
-        float u = good ? U / Wd + w.pp.x : 0.0f, v = good ? Vv / Wd + w.pp.y : 0.0f;
-        umin = umax = u;
-        vmin = vmax = v;
-      }
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-        umin = fminf(umin, __shfl_xor_sync(0xffffffffu, umin, o));
-        umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, o));
-        vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
-        vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-        good &= __shfl_xor_sync(0xffffffffu, good, o);
-      }
-      if (vi < nvc && cr == 0) {
-        int4 t = make_int4(0, 0, FP_GLOBAL, TB_BWW);
-        if (good && fabsf(umin) < 1e6f && fabsf(umax) < 1e6f && fabsf(vmin) < 1e6f &&
-            fabsf(vmax) < 1e6f) {
-          int x0 = (int)floorf(umin) - 1, x1 = (int)floorf(umax) + 2;
-          int r0 = (int)floorf(vmin) - 1, r1 = (int)floorf(vmax) + 2;
-          if (x1 < 0 || x0 >= a.W || r1 < 0 || r0 >= a.H)
-            t = make_int4(x0, r0, FP_SKIP, 0);
-          else if (r1 - r0 + 1 <= TB_BH && x1 - x0 + 1 <= TB_BWW)
-            t = make_int4(x0, r0, FP_WIDE, (x1 - x0 + 1) | ((r1 - r0 + 1) << 8));
-        }
-        vtab[vi] = t;
-      }
-    }
-    __syncthreads();
-    for (int vi = 0; vi < nvc; ++vi) {
-      int4 t = vtab[vi];
-      if (t.z == FP_SKIP) continue;
-      const dc::BPView w = sv[vi];
-      float *img = gbase + (size_t)(c0 + vi) * np;
-      float U0 = fmaf(w.r0.x, xo, fmaf(w.r0.y, yo, fmaf(w.r0.z, zo, w.r0.w)));
-      float V0 = fmaf(w.r1.x, xo, fmaf(w.r1.y, yo, fmaf(w.r1.z, zo, w.r1.w)));
-      float W0 = fmaf(w.r2.x, xo, fmaf(w.r2.y, yo, fmaf(w.r2.z, zo, w.r2.w)));
-      float dU = w.r0.z * a.dz, dV = w.r1.z * a.dz, dW = w.r2.z * a.dz;
-      float ex = w.ca.x + xo, ey = w.ca.y + yo, ez0 = w.ca.z + zo;
-      float rho2 = fmaf(ex, ex, ey * ey);
-      // fixed-point unit of this (box, view); CTA-uniform
-      float dcx = w.ca.x + bcx, dcy = w.ca.y + bcy, dcz = w.ca.z + bcz;
-      float dmin = sqrtf(dcx * dcx + dcy * dcy + dcz * dcz) - bhd;
-      if (t.z == FP_WIDE && !(dmin > 1.0f)) t.z = FP_GLOBAL;
-      if (t.z == FP_WIDE) {
-        const float bound = gsum / (dmin * dmin);             // >= any pixel sum
-        const float to_fix = 1073741824.0f / bound;            // bound -> 2^30
-        const float from_fix = bound * (1.0f / 1073741824.0f);
-        const float cul = w.pp.x - (float)t.x, cvl = w.pp.y - (float)t.y;
-        const float umx = (float)TB_BWW - 1.001f, vmx = (float)TB_BH - 1.001f;
-        int *tile = tiles[cur];
-        auto scatter = [&](auto to_int) {
-#pragma unroll
-          for (int k = 0; k < TB_NZ; ++k) {
-            if (gv[k] == 0.0f) continue;
-            float kf = rotf + (float)k;  // voxel (k + rot) mod TB_NZ
-            kf = (kf >= (float)TB_NZ) ? kf - (float)TB_NZ : kf;
-            float rw = dc::rcp_approx(fmaf(kf, dW, W0));
-            float u = fminf(fmaxf(fmaf(fmaf(kf, dU, U0), rw, cul), 0.0f), umx);
-            float v = fminf(fmaxf(fmaf(fmaf(kf, dV, V0), rw, cvl), 0.0f), vmx);
-            float ez = fmaf(kf, a.dz, ez0);
-            float gk = gv[k] * dc::rcp_approx(fmaf(ez, ez, rho2)) * to_fix;
-            float fu, fv;
-            int j = dc::floor_frac(u, fu), r = dc::floor_frac(v, fv);
-            int *p = tile + r * TA_S + j;
-            float g1 = gk * fv, g0 = gk - g1;
-            float g01 = g0 * fu, g11 = g1 * fu;
-            atomicAdd(p, to_int(g0 - g01));
-            atomicAdd(p + 1, to_int(g01));
-            atomicAdd(p + TA_S, to_int(g1 - g11));
-            atomicAdd(p + TA_S + 1, to_int(g11));
-          }
-        };
-        if (any) {
-          if (magic_round)
-            scatter([](float x) {
-              return __float_as_int(__fadd_rn(x, 12582912.0f)) - 0x4B400000;  // |x| < 2^22
-            });
-          else
-            scatter([](float x) { return __float2int_rn(x); });
-        }
-        // the previous view's tile (complete since the last barrier) to g^F's
-        // gradient, cleared for the view after this one
-        if (pending) flush_pending();
-        __syncthreads();
-        pending = true;
-        pt = t;
-        p_from_fix = from_fix;
-        p_img = img;
-        cur ^= 1;
-      } else if (any) {
-#pragma unroll
-        for (int k = 0; k < TB_NZ; ++k) {
-          if (gv[k] == 0.0f) continue;
-          float kf = rotf + (float)k;  // voxel (k + rot) mod TB_NZ
-          kf = (kf >= (float)TB_NZ) ? kf - (float)TB_NZ : kf;
-          float dep = fmaf(kf, dW, W0);
-          if (!(dep > 0.0f)) continue;
-          float rw = __frcp_rn(dep);
-          float u = fmaf(fmaf(kf, dU, U0), rw, w.pp.x);
-          float v = fmaf(fmaf(kf, dV, V0), rw, w.pp.y);
-          float ez = fmaf(kf, a.dz, ez0);
-          float g = gv[k] * __frcp_rn(fmaf(ez, ez, rho2));
-          u = fminf(fmaxf(u, -2.0f), (float)a.W + 1.0f);
-          v = fminf(fmaxf(v, -2.0f), (float)a.H + 1.0f);
-          float fu, fv;
-          int j = dc::floor_frac(u, fu), r = dc::floor_frac(v, fv);
-          bool j0 = (j >= 0 && j < a.W), j1 = (j + 1 >= 0 && j + 1 < a.W);
-          bool r0 = (r >= 0 && r < a.H), r1 = (r + 1 >= 0 && r + 1 < a.H);
-          float *p = img + (ptrdiff_t)r * a.W + j;
-          if (r0 && j0) atomicAdd(p, g * (1.0f - fu) * (1.0f - fv));
-          if (r0 && j1) atomicAdd(p + 1, g * fu * (1.0f - fv));
-          if (r1 && j0) atomicAdd(p + a.W, g * (1.0f - fu) * fv);
-          if (r1 && j1) atomicAdd(p + a.W + 1, g * fu * fv);
-        }
-      }
-    }
-  }
-  if (pending) flush_pending();  // its scatter ended at the last barrier
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -773,46 +430,6 @@ int dc_backproject(const dc_geometry *g, int B, const void *gF, int dtype,
       return dc::fail(DC_ERR_ARG, "dc_backproject: unknown dtype");
   }
   DC_CHECK_LAUNCH("k_bp3d");
-  return DC_OK;
-}
-
-int dc_backproject_adjoint(const dc_geometry *g, int B, const float *grad_vol,
-                           const float *relu_vol, float *grad_gF, void *stream) {
-  int rc = check_bp(g, B, "dc_backproject_adjoint");
-  if (rc) return rc;
-  if (!grad_vol || !grad_gF)
-    return dc::fail(DC_ERR_ARG, "dc_backproject_adjoint: NULL grad_vol or grad_gF");
-  const dc_geometry_desc &d = g->d;
-  cudaStream_t st = (cudaStream_t)stream;
-  DC_CUDA(cudaMemsetAsync(grad_gF, 0,
-                          sizeof(float) * (size_t)B * d.n_views * d.det_rows * d.det_cols, st));
-  BPAdjArgs a;
-  a.grad_vol = grad_vol;
-  a.relu_vol = relu_vol;
-  a.views = g->bpv;
-  a.grad_gF = grad_gF;
-  a.V = d.n_views;
-  a.H = d.det_rows;
-  a.W = d.det_cols;
-  a.nx = d.vol_x;
-  a.ny = d.vol_y;
-  a.nz = d.vol_z;
-  a.B = B;
-  a.dx = (float)d.voxel[0];
-  a.dy = (float)d.voxel[1];
-  a.dz = (float)d.voxel[2];
-  dim3 blk(BP_TX, BP_TY);
-  dim3 grid((d.vol_x + BP_TX - 1) / BP_TX, (d.vol_y + BP_TY - 1) / BP_TY,
-            ((d.vol_z + BP_NZ - 1) / BP_NZ) * B);
-  dc::ProfScope ps(dc::KID_BP3D_ADJ, st);
-  if (getenv("DC_BP_ADJ_GLOBAL")) {
-    k_bp3d_adj<<<grid, blk, 0, st>>>(a);
-  } else {
-    dim3 gridt((d.vol_x + TB_TX - 1) / TB_TX, (d.vol_y + TB_TY - 1) / TB_TY,
-               ((d.vol_z + TB_NZ - 1) / TB_NZ) * B);
-    k_bp3d_adj_tile<<<gridt, blk, 0, st>>>(a);
-  }
-  DC_CHECK_LAUNCH("k_bp3d_adj");
   return DC_OK;
 }
 

@@ -69,3 +69,19 @@ def test_box_depth_of_the_geometry(voxel, n, nz, depth):
     tile or are fewer than the SMs."""
     gg, _ = _problem("circle", 8, 64, 64, n, nz, voxel, pitch=1.5)
     assert api.dc_geometry_get_tuning(gg)["bp_nz"] == depth
+
+
+# rows of whole quads and not, detectors narrower than the projected volume,
+# volumes smaller than a box, one voxel beyond it and of whole boxes
+@pytest.mark.parametrize("W", [40, 41, 42])
+@pytest.mark.parametrize("n,nz", [(7, 5), (17, 33), (32, 32), (21, 15)])
+@pytest.mark.parametrize("relu", [False, True])
+def test_adjoint_at_edges(W, n, nz, relu):
+    gg, og = _problem("sinusoid", 34, 30, W, n, nz, 2.4)
+    rng = np.random.default_rng(W * n)
+    gv = rng.normal(size=(2, nz, n, n)).astype(np.float32)
+    vol = rng.normal(size=gv.shape).astype(np.float32)
+    got = api.dc_backproject_adjoint(gg, torch.as_tensor(gv, device="cuda"),
+                                     torch.as_tensor(vol, device="cuda") if relu else None)
+    ref = orc.backproject_adjoint(og, gv * (vol > 0) if relu else gv)
+    assert rel_l2(got.double().cpu().numpy(), ref) < 1e-5
