@@ -113,11 +113,27 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 2) k_bp3d_tma(BPArgs a, unsigned
     dc::fence_barrier_init();
   }
   __syncthreads();
-  unsigned it = 0;
-  if (!bp_box<T, KAHAN, NZ>(a, a.vol, &tmn, &tmw, err, blockIdx.x, blockIdx.y, blockIdx.z, dsm,
-                            full, sv, vtab, it)) {
+  if (!bp_layer_box<T, KAHAN, NZ, LD_TMA>(a, &tmn, &tmw, err, dsm, full, sv, vtab)) {
     for (int q = 0; q < TB_NS; ++q) dc::mbar_wait_bounded(&full[q], 0, nullptr);
   }
+}
+
+// views split over the CTAs of a cluster (bp_split_box); 16-deep boxes
+template <typename T, bool KAHAN>
+__global__ void __launch_bounds__(TB_TX *TB_TY, 2)
+    k_bp3d_split(BPArgs a, unsigned *err, int split, const __grid_constant__ CUtensorMap tmn,
+                 const __grid_constant__ CUtensorMap tmw) {
+  extern __shared__ __align__(128) unsigned char dsm[];
+  __shared__ uint64_t full[TB_NS];
+  __shared__ dc::BPView sv[TB_VCH];
+  __shared__ int4 vtab[TB_VCH];
+  __shared__ int good;
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    for (int q = 0; q < TB_NS; ++q) dc::mbar_init(&full[q], 1);
+    dc::fence_barrier_init();
+  }
+  __syncthreads();
+  bp_split_box<T, KAHAN, 16, LD_TMA>(a, &tmn, &tmw, err, split, dsm, full, sv, vtab, &good);
 }
 
 // Persistent backprojection of a batch of problems (orbits of uneven view
@@ -221,6 +237,16 @@ bool make_map(CUtensorMap *m, const void *base, int dtype, int W, int H, long lo
 template <typename T, int NZ>
 int launch_bp_tma_nz(const dc_geometry *g, BPArgs &a, bool kahan, cudaStream_t st,
                      const CUtensorMap &mn, const CUtensorMap &mw) {
+  if (g->bp_split > 1 && NZ == 16) {
+    auto kernel = kahan ? k_bp3d_split<T, true> : k_bp3d_split<T, false>;
+    DC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)bp_smem<T>()));
+    dim3 grid((a.nx + TB_TX - 1) / TB_TX, (a.ny + TB_TY - 1) / TB_TY,
+              ((a.z_end - a.z_begin + 15) / 16) * a.B);
+    DC_CUDA(launch_split(kernel, grid, bp_smem<T>(), st, g->bp_split, a, g->w_flags, g->bp_split,
+                         mn, mw));
+    return DC_OK;
+  }
   dim3 blk(TB_TX, TB_TY);
   dim3 grid((a.nx + TB_TX - 1) / TB_TX, (a.ny + TB_TY - 1) / TB_TY,
             ((a.z_end - a.z_begin + NZ - 1) / NZ) * a.B);
@@ -252,24 +278,8 @@ int launch_bp_tma(const dc_geometry *g, BPArgs &a, int dtype, bool kahan, cudaSt
   if (!make_map(&mn, a.gF, dtype, a.W, a.H, nimg, TileShape<T>::BWN) ||
       !make_map(&mw, a.gF, dtype, a.W, a.H, nimg, TileShape<T>::BWW))
     return DC_OK;
-  // with 32-deep boxes, a last layer of at most 16 planes takes 16-deep ones
-  // (half the work, and a footprint of its own size)
-  const int tail = (g->bp_nz == 32) ? (a.z_end - a.z_begin) % 32 : 0;
-  const int z_end = a.z_end;
-  int rc = DC_OK;
-  if (tail > 0 && tail <= 16) {
-    BPArgs t = a;
-    t.z_begin = z_end - tail;
-    if ((rc = launch_bp_tma_nz<T, 16>(g, t, kahan, st, mn, mw))) return rc;
-    if (a.z_begin < z_end - tail) {
-      DC_CHECK_LAUNCH("k_bp3d_tma");
-      a.z_end = z_end - tail;
-      rc = launch_bp_tma_nz<T, 32>(g, a, kahan, st, mn, mw);
-    }
-  } else {
-    rc = (g->bp_nz == 16) ? launch_bp_tma_nz<T, 16>(g, a, kahan, st, mn, mw)
-                          : launch_bp_tma_nz<T, 32>(g, a, kahan, st, mn, mw);
-  }
+  int rc = (g->bp_nz == 16) ? launch_bp_tma_nz<T, 16>(g, a, kahan, st, mn, mw)
+                            : launch_bp_tma_nz<T, 32>(g, a, kahan, st, mn, mw);
   if (rc) return rc;
   *used = true;
   return DC_OK;
@@ -380,6 +390,14 @@ void bp_plan(dc_geometry *g) {
   const long boxes = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
                      ((d.vol_z + TB_NZ - 1) / TB_NZ);
   g->bp_nz = (fit < all * 0.95 || boxes < 152) ? 16 : 32;
+  // views split over clusters where 16-deep boxes are fewer than the SMs: as
+  // many CTAs as two per SM hold, at least 8 views each (64 boxes, 64 views:
+  // 57 us unsplit, 33 us split by four)
+  const long boxes16 = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
+                       ((d.vol_z + 15) / 16);
+  g->bp_split = 1;
+  while (g->bp_split < 8 && 2 * g->bp_split * boxes16 <= 304 && d.n_views >= 16 * g->bp_split)
+    g->bp_split *= 2;
 }
 
 }  // namespace dc

@@ -128,7 +128,7 @@ __device__ __forceinline__ void red_add4(unsigned addr, int i00, int i01, int i1
 }
 
 template <bool VEC4>
-__global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a) {
+__global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, int split) {
   __shared__ __align__(16) int tiles[2][TB_BH * TA_S];
   __shared__ dc::BPView sv[TB_VCH];
   __shared__ int4 vtab[TB_VCH];
@@ -136,11 +136,14 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a) 
   __shared__ float wmax[TB_TX * TB_TY / 32];
   const int tid = threadIdx.y * TB_TX + threadIdx.x;
   const int zblocks = (a.nz + TB_NZ - 1) / TB_NZ;
-  const int b = blockIdx.z / zblocks;
+  // blockIdx.z = box * split + share of the views
+  const int bz = blockIdx.z / split, part = blockIdx.z % split, b = bz / zblocks;
+  const int v_begin = (int)((long long)a.V * part / split),
+            v_end = (int)((long long)a.V * (part + 1) / split);
   // full boxes: one at the volume's end is moved back inside and takes the
   // gradients of its own voxels only (see bp_box)
   const int x_own = blockIdx.x * TB_TX, y_own = blockIdx.y * TB_TY;
-  const int z_own = (blockIdx.z % zblocks) * TB_NZ;
+  const int z_own = (bz % zblocks) * TB_NZ;
   const int x0b = max(min(x_own, a.nx - TB_TX), 0), y0b = max(min(y_own, a.ny - TB_TY), 0);
   const int z0 = max(min(z_own, a.nz - TB_NZ), 0);
   const int ix = x0b + threadIdx.x, iy = y0b + threadIdx.y;
@@ -258,8 +261,8 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a) 
     }
   };
 
-  for (int c0 = 0; c0 < a.V; c0 += TB_VCH) {
-    const int nvc = min(TB_VCH, a.V - c0);
+  for (int c0 = v_begin; c0 < v_end; c0 += TB_VCH) {
+    const int nvc = min(TB_VCH, v_end - c0);
     __syncthreads();
     {  // footprints: thread = (view, corner), as in the forward kernel
       const int vi = tid >> 3, cr = tid & 7;
@@ -460,11 +463,18 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
   } else {
     dim3 gridt((d.vol_x + TB_TX - 1) / TB_TX, (d.vol_y + TB_TY - 1) / TB_TY,
                ((d.vol_z + TB_NZ - 1) / TB_NZ) * B);
+    // few boxes share their views among CTAs (a view's gradient is summed by
+    // atomics anyway), up to the three CTAs that an SM holds and down to 8
+    // views each
+    const long boxes = (long)gridt.x * gridt.y * gridt.z;
+    int split = 1;
+    while (split < 16 && 2 * split * boxes <= 456 && d.n_views >= 16 * split) split *= 2;
+    gridt.z *= split;
     // float4 atomics need 16-byte pixel quads
     if ((a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0)
-      k_bp3d_adj_tile<true><<<gridt, blk, 0, st>>>(a);
+      k_bp3d_adj_tile<true><<<gridt, blk, 0, st>>>(a, split);
     else
-      k_bp3d_adj_tile<false><<<gridt, blk, 0, st>>>(a);
+      k_bp3d_adj_tile<false><<<gridt, blk, 0, st>>>(a, split);
   }
   DC_CHECK_LAUNCH("k_bp3d_adj");
   return DC_OK;

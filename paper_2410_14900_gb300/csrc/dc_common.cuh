@@ -151,6 +151,7 @@ struct dc_geometry {
   int chunk_capacity;        // images the work area was sized for
   int l2_images;             // images whose per-image work area stays in L2
   int bp_nz;                 // voxels per thread along z in the backprojector (16, 32)
+  int bp_split;              // CTAs (a cluster) that share the views of a 16-deep box
   size_t img_stride;         // floats per padded image  (H * Wp)
   size_t sino_stride;        // floats per padded sinogram (n_mu * NSp)
   int Wp, NSp;               // padded row lengths (multiples of 4)
@@ -212,7 +213,7 @@ int backproject_slab(const dc_geometry *g, int B, const void *gF, int dtype,
 int backproject_rows(const dc_geometry *g, int B, const void *gF, int dtype,
                      const float *gF_scale, float *vol, unsigned flags, int z_begin, int z_end,
                      cudaStream_t st, bool *used);
-// the backprojection's box depth for this geometry (g->bp_nz)
+// the backprojection's box depth and view split for this geometry
 void bp_plan(dc_geometry *g);
 // the batched persistent filter (dc_filter.cu): one launch filters every
 // view of up to 32 problems into the given g^F buffers (and FP16 scales)
