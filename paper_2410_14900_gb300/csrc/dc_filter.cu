@@ -1246,14 +1246,33 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 
 namespace dc {
 
+// Images that the work area holds.  The per-image kernels want a chunk that
+// stays in the 126 MB L2 (112 MB); the four-image kernels take few CTAs per
+// image, so larger chunks keep the last wave of a launch small (their L2
+// working set is the few images in flight).  The autotuner may use fewer
+// images per chunk.
+static int chunk_capacity(const dc_geometry *g) {
+  const dc_geometry_desc &d = g->d;
+  const size_t img = (size_t)d.det_rows * round4(d.det_cols), sino = (size_t)d.n_mu * round4(d.n_s);
+  const size_t per_img = ((g->quad ? 2 : 1) * img + 2 * sino) * sizeof(float);
+  const long target = (g->quad ? 384L : 112L) << 20;
+  const char *env = getenv("DC_CHUNK_IMAGES");
+  int ci = env ? atoi(env) : (int)(target / (long)per_img);
+  if (ci < 4) ci = 4;
+  if (ci > 256) ci = 256;
+  return g->quad ? ci & ~3 : ci;
+}
+
 // The four-image line sums share every sample position, so all views need
 // the same principal point.  Matrices of one scanner give it up to the
 // rounding of their recovery (~1e-10 pixels); 1e-8 pixels is below a
 // hundredth of the FP32 positions' own rounding (~1e-6), and a detector
 // calibrated view by view differs by far more and keeps the per-image
 // kernel, as do rows too long for two stages.  The angles per group are the
-// number with the least time per angle: rounds of a CTA's warps over its
-// tasks, plus half a round for set-up and epilogue.
+// number with the least time for a chunk: waves of CTAs (one per SM) times a
+// CTA's rounds of its warps over its tasks plus its set-up and epilogue, 8 us
+// against 0.69 us per band and round (64 views of 64 x 64, 180 x 64 lines: 48
+// us in two waves of up to 16 angles, 38 us in one of 23).
 int quad_plan(dc_geometry *g) {
   const dc_geometry_desc &d = g->d;
   g->quad = 0;
@@ -1264,10 +1283,22 @@ int quad_plan(dc_geometry *g) {
         return DC_OK;
   const int nch = (d.n_s + 31) / 32, NSp = round4(d.n_s);
   const L4Shape sh = l4_shape(d.det_rows, d.det_cols);
+  const int nb[2] = {(d.n_mu + 1) / 2, d.n_mu / 2};  // angles per branch, within one
+  g->quad = 1;
+  const int quads = (std::min(d.n_views, chunk_capacity(g)) + 3) / 4;
+  g->quad = 0;
+  const double over = 23.2 * L4_RB / (d.det_rows + d.det_cols);
   double best = 0.0;
-  for (int mg = 1; mg <= DC_LS_MAX_MG && mg * nch <= L4_TASKS; ++mg) {
+  for (int mg = 1; mg <= L4_MAX_MG && mg * nch <= L4_TASKS; ++mg) {
     if (l4_smem(sh, mg, NSp) > L4_SMEM_BUDGET) break;
-    const double cost = ((mg * nch + L4_WARPS - 1) / L4_WARPS + 0.5) / mg;
+    int groups = 0, most = 0;
+    for (int br = 0; br < 2; ++br) {
+      const int ng = (nb[br] + mg - 1) / mg;
+      groups += ng;
+      if (ng) most = std::max(most, (nb[br] + ng - 1) / ng);
+    }
+    const int rounds = (most * nch + L4_WARPS - 1) / L4_WARPS;
+    const double cost = ((groups * quads + 151) / 152) * (rounds + over);
     if (!g->quad || cost < best) {
       best = cost;
       g->q_mg = mg;
@@ -1283,17 +1314,7 @@ int alloc_workspace(dc_geometry *g) {
   g->NSp = round4(d.n_s);
   g->img_stride = (size_t)d.det_rows * g->Wp;
   g->sino_stride = (size_t)d.n_mu * g->NSp;
-  size_t per_img = ((g->quad ? 2 : 1) * g->img_stride + 2 * g->sino_stride) * sizeof(float);
-  // The per-image kernels want a chunk that stays in the 126 MB L2 (112 MB);
-  // the four-image kernels take few CTAs per image, so larger chunks keep the
-  // last wave of a launch small (their L2 working set is the few images in
-  // flight).  The autotuner may use fewer images per chunk than it holds.
-  long target = (g->quad ? 384L : 112L) << 20;
-  const char *env = getenv("DC_CHUNK_IMAGES");
-  int ci = env ? atoi(env) : (int)(target / (long)per_img);
-  if (ci < 4) ci = 4;
-  if (ci > 256) ci = 256;
-  if (g->quad) ci &= ~3;
+  const int ci = chunk_capacity(g);
   g->l2_images = std::max(4, (int)((112L << 20) /
                                    (long)((g->img_stride + 2 * g->sino_stride) * sizeof(float))));
   g->chunk_images = ci;

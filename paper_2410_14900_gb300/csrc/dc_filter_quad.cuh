@@ -30,11 +30,12 @@ constexpr int L4_WARPS = 19;
 constexpr int L4_THREADS = 32 * L4_WARPS + 32;
 constexpr int L4_T = 6;                  // tasks (angle, 32 lines) per warp
 constexpr int L4_TASKS = L4_WARPS * L4_T;
+constexpr int L4_MAX_MG = 32;            // angles per group
 constexpr int L4_RB = 8;                 // steps per band
 // a line that meets the detector in a band moves at most 7 samples in it:
 // taps lie in [-8, len + 8]
 constexpr int L4_PJ = 9;
-constexpr int L4_SMEM_BUDGET = 225 * 1024;
+constexpr int L4_SMEM_BUDGET = 222 * 1024;  // beside 4 KB of static tables
 
 // staging of one band: nbox TMA boxes of boxh samples x 8 steps x 4 images
 struct L4Shape {
@@ -69,28 +70,37 @@ __global__ void __launch_bounds__(256) k_prep4(PrepArgs a, float4 *__restrict__ 
                                                float4 *__restrict__ cols) {
   __shared__ float4 tile[32][33];
   const int grp = blockIdx.z;
-  const int j = blockIdx.x * 32 + threadIdx.x;
-  for (int q = threadIdx.y; q < 32; q += 8) {
-    const int r = blockIdx.y * 32 + q;
-    if (r >= a.H || j >= a.W) continue;
-    float val[4];
+  const int j = blockIdx.x * 32 + threadIdx.x, rb = blockIdx.y * 32 + threadIdx.y;
+  float val[4][4];  // [row rb + 8 p][image], all loads in flight together
+  const float *src[4];
+  dc::FView f[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int n = 4 * grp + i;
-      val[i] = 0.0f;
-      if (n < a.n_img) {
-        const int v = a.v0 + n / a.B, b = a.b0 + n % a.B;
-        val[i] = a.src[(((size_t)b * a.V + v) * a.H + r) * a.W + j];
-        if (a.weight != WT_NONE) {
-          const dc::FView f = a.fv[v];
-          const float x = (j - f.cu) * a.pitch, y = (r - f.cv) * a.pitch;
-          const float l2 = fmaf(x, x, fmaf(y, y, f.D * f.D));
-          val[i] *= (a.weight == WT_COS) ? f.D * rsqrtf(l2) : l2;
-        }
+  for (int i = 0; i < 4; ++i) {
+    const int n = min(4 * grp + i, a.n_img - 1), v = a.v0 + n / a.B, b = a.b0 + n % a.B;
+    src[i] = a.src + ((size_t)b * a.V + v) * a.H * a.W + j;
+    f[i] = a.fv[v];
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      val[p][i] = (4 * grp + i < a.n_img && rb + 8 * p < a.H && j < a.W)
+                      ? src[i][(size_t)(rb + 8 * p) * a.W]
+                      : 0.0f;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int r = rb + 8 * p;
+    if (r >= a.H || j >= a.W) continue;
+    if (a.weight != WT_NONE) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float x = (j - f[i].cu) * a.pitch, y = (r - f[i].cv) * a.pitch;
+        const float l2 = fmaf(x, x, fmaf(y, y, f[i].D * f[i].D));
+        val[p][i] *= (a.weight == WT_COS) ? f[i].D * rsqrtf(l2) : l2;
       }
     }
-    const float4 v4 = make_float4(val[0], val[1], val[2], val[3]);
-    tile[q][threadIdx.x] = v4;
+    const float4 v4 = make_float4(val[p][0], val[p][1], val[p][2], val[p][3]);
+    tile[threadIdx.y + 8 * p][threadIdx.x] = v4;
     rows[((size_t)grp * a.H + r) * a.W + j] = v4;
   }
   __syncthreads();
@@ -124,9 +134,9 @@ __global__ void __launch_bounds__(L4_THREADS, 1)
                const __grid_constant__ CUtensorMap tm_rows) {
   constexpr bool DIFF = (MODE != M_RAW);
   extern __shared__ __align__(1024) unsigned char dyn[];
-  __shared__ LineMu lmu[dc::DC_LS_MAX_MG];
-  __shared__ dc::MuRec lcs[dc::DC_LS_MAX_MG];
-  __shared__ int lm[dc::DC_LS_MAX_MG];
+  __shared__ LineMu lmu[L4_MAX_MG];
+  __shared__ dc::MuRec lcs[L4_MAX_MG];
+  __shared__ int lm[L4_MAX_MG];
   __shared__ dc::FView fvs[4];
   __shared__ uint64_t full[2], empty[2];
 
@@ -658,6 +668,9 @@ __global__ void __launch_bounds__(B4_THREADS, RY == 8 ? 2 : 4)
   for (; c < nchunk; ++c) {
     if (!dc::mbar_wait_bounded(&full[c & 1], (c >> 1) & 1, a.err)) ok = false;
     const int nm = min(B4_MC, a.n_mu - c * B4_MC);
+    // few pixels per thread: several angles in flight hide the chain from an
+    // angle's constants to its taps
+#pragma unroll(RY == 2 ? 4 : 1)
     for (int mi = 0; mi < nm; ++mi) {
       const B4Mu M = bmu[c & 1][mi];
       const unsigned cb = M.cbase + sbase;
