@@ -39,7 +39,7 @@ class DefriseClackFunction(torch.autograd.Function):
         if cache_s and need_grad:
             S = torch.empty((g.shape[0], geom.V) + geom.sino_shape, device=g.device,
                             dtype=torch.float32)
-        gF, _ = api.dc_filter(geom, g, Wc, S_out=S)
+        gF, _ = api.dc_filter(geom, g, Wc, api.transient_dtype(geom, g.shape[0]), S_out=S)
         vol = api.dc_backproject(geom, gF, relu=relu)
         del gF
         ctx.geom = geom

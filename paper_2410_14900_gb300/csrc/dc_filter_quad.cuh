@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(B4_THREADS, RY == 8 ? 2 : 4)
     const int nm = min(B4_MC, a.n_mu - c * B4_MC);
     // few pixels per thread: several angles in flight hide the chain from an
     // angle's constants to its taps
-#pragma unroll(RY == 2 ? 4 : 1)
+#pragma unroll(RY == 2 ? 4 : 2)
     for (int mi = 0; mi < nm; ++mi) {
       const B4Mu M = bmu[c & 1][mi];
       const unsigned cb = M.cbase + sbase;
