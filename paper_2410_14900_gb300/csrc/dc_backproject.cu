@@ -389,7 +389,8 @@ void bp_plan(dc_geometry *g) {
   }
   const long boxes = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
                      ((d.vol_z + TB_NZ - 1) / TB_NZ);
-  g->bp_nz = (fit < all * 0.95 || boxes < 152) ? 16 : 32;
+  g->bp_fit32 = fit >= all * 0.95;
+  g->bp_nz = (!g->bp_fit32 || boxes < 152) ? 16 : 32;
   // views split over clusters where 16-deep boxes are fewer than the SMs: as
   // many CTAs as two per SM hold, at least 8 views each (64 boxes, 64 views:
   // 57 us unsplit, 33 us split by four)

@@ -104,17 +104,19 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_bp3d_adj(BPAdjArgs a) {
 //
 // Bound by the shared atomics: a bare loop of four per voxel runs at 8.1e11
 // voxels/s, 29.8 ms for 4 x 256^3 voxels and 360 views.  With 55 instructions
-// per voxel (and a branch for its zero gradient) that took 44.9 ms; two voxels
-// of a column (k and k + 16) stepped together in packed FP32x2, without clamps
-// (full boxes, as in the forward kernel) and without branches take 30
-// instructions, and with float4 atomics into g^F's gradient (scalar ones: 5 ms
-// more) and three CTAs per SM (two: 33.1) 32.2 ms.  Merging a column's
-// consecutive voxels, which mostly share a detector row, saves up to half of
-// the atomics but wants the others predicated: 43 to 52 ms.
+// per voxel that took 44.9 ms; two voxels of a column stepped together in packed
+// FP32x2, without clamps (full boxes, as in the forward kernel), take 30
+// instructions; with float4 atomics into g^F's gradient (scalar ones: 5 ms
+// more) and three CTAs per SM (two: 0.5 to 1 ms more) 32.2 ms, and without the
+// atomics of zero gradients (half of the voxels there, behind the ReLU) 30.1 ms.
+// Merging a column's consecutive voxels, which mostly share a detector row,
+// saves up to half of the atomics but wants the others predicated: 43 to 52 ms.
+//
+// Boxes are 32 deep, or 16 where 32-deep ones mostly do not fit the tile and
+// would scatter into global memory (214^2 x 178 voxels of 1.4 pixels, 86 views:
+// 5.2 ms, here 1.3).
 constexpr int TA_S = 68;  // row stride: 16-byte rows (69: 34.0 ms)
-constexpr int TA_K = TB_NZ / 2;
 static_assert(TA_S >= TB_BWW + 3, "a tile row holds the widest footprint from an aligned column");
-static_assert(TB_NZ == 32 && TA_K == 16, "the voxel order is rotated by the lane in 16 steps");
 
 // four taps: pixel pairs at addr and one tile row below
 __device__ __forceinline__ void red_add4(unsigned addr, int i00, int i01, int i10, int i11) {
@@ -127,15 +129,16 @@ __device__ __forceinline__ void red_add4(unsigned addr, int i00, int i01, int i1
       : "memory");
 }
 
-template <bool VEC4>
+template <bool VEC4, int NZ>
 __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, int split) {
+  constexpr int NH = NZ / 2;  // a step takes voxels NH apart
   __shared__ __align__(16) int tiles[2][TB_BH * TA_S];
   __shared__ dc::BPView sv[TB_VCH];
   __shared__ int4 vtab[TB_VCH];
   __shared__ float wsum[TB_TX * TB_TY / 32];
   __shared__ float wmax[TB_TX * TB_TY / 32];
   const int tid = threadIdx.y * TB_TX + threadIdx.x;
-  const int zblocks = (a.nz + TB_NZ - 1) / TB_NZ;
+  const int zblocks = (a.nz + NZ - 1) / NZ;
   // blockIdx.z = box * split + share of the views
   const int bz = blockIdx.z / split, part = blockIdx.z % split, b = bz / zblocks;
   const int v_begin = (int)((long long)a.V * part / split),
@@ -143,9 +146,9 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
   // full boxes: one at the volume's end is moved back inside and takes the
   // gradients of its own voxels only (see bp_box)
   const int x_own = blockIdx.x * TB_TX, y_own = blockIdx.y * TB_TY;
-  const int z_own = (bz % zblocks) * TB_NZ;
+  const int z_own = (bz % zblocks) * NZ;
   const int x0b = max(min(x_own, a.nx - TB_TX), 0), y0b = max(min(y_own, a.ny - TB_TY), 0);
-  const int z0 = max(min(z_own, a.nz - TB_NZ), 0);
+  const int z0 = max(min(z_own, a.nz - NZ), 0);
   const int ix = x0b + threadIdx.x, iy = y0b + threadIdx.y;
   const float cx = 0.5f * (float)(a.nx - 1), cy = 0.5f * (float)(a.ny - 1),
               cz = 0.5f * (float)(a.nz - 1);
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
   const float zo = ((float)z0 - cz) * a.dz;
   const float bx0 = ((float)x0b - cx) * a.dx, bx1 = ((float)(x0b + TB_TX - 1) - cx) * a.dx;
   const float by0 = ((float)y0b - cy) * a.dy, by1 = ((float)(y0b + TB_TY - 1) - cy) * a.dy;
-  const float bz0 = zo, bz1 = ((float)(z0 + TB_NZ - 1) - cz) * a.dz;
+  const float bz0 = zo, bz1 = ((float)(z0 + NZ - 1) - cz) * a.dz;
   // box centre and half-diagonal (for the distance bound)
   const float bcx = 0.5f * (bx0 + bx1), bcy = 0.5f * (by0 + by1), bcz = 0.5f * (bz0 + bz1);
   const float bhd = 0.5f * sqrtf((bx1 - bx0) * (bx1 - bx0) + (by1 - by0) * (by1 - by0) +
@@ -162,23 +165,23 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
   const size_t np = (size_t)a.H * a.W;
   const size_t nvox = (size_t)a.nx * a.ny * a.nz;
   const bool own = ix >= x_own && ix < a.nx && iy >= y_own && iy < a.ny;
-  // Step k takes the column's voxels kz and kz + 16 with kz = (k + lane) mod
-  // 16, the upper half-warp in the other order: at each step the lanes of a
-  // warp are at 32 different depths, so lanes whose columns project to the same
+  // Step k takes the column's voxels kz and kz + NH with kz = (k + lane) mod NH,
+  // every second NH lanes in the other order: at each step NZ neighbouring lanes
+  // are at NZ different depths, so lanes whose columns project to the same
   // detector column (columns lined up with the view direction) hit different
   // detector rows.  The fixed-point sums are exact, so the order does not
   // change the result.
-  const int rot = tid & 15, off = tid & 16;
-  const float flip = off ? -16.0f : 16.0f;
-  float2 gv[TA_K];
+  const int rot = tid & (NH - 1), off = tid & NH;
+  const float flip = off ? -(float)NH : (float)NH;
+  float2 gv[NH];
   float gs = 0.0f, gm = 0.0f;
 #pragma unroll
-  for (int k = 0; k < TA_K; ++k) {
-    const int kz = ((k + rot) & 15) + off;
+  for (int k = 0; k < NH; ++k) {
+    const int kz = ((k + rot) & (NH - 1)) + off;
     float g[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int iz = z0 + (kz ^ (16 * h));
+      const int iz = z0 + (kz ^ (NH * h));
       g[h] = 0.0f;
       if (own && iz >= z_own && iz < a.nz) {
         const size_t o = (size_t)b * nvox + ((size_t)iz * a.ny + iy) * a.nx + ix;
@@ -339,10 +342,10 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
         auto scatter = [&](auto magic) {
           float kf = (float)(rot + off);
 #pragma unroll
-          for (int k = 0; k < TA_K; ++k) {
-            const float2 kf2 = make_float2(kf, kf + flip);  // voxels kz, kz ^ 16
+          for (int k = 0; k < NH; ++k) {
+            const float2 kf2 = make_float2(kf, kf + flip);  // voxels kz, kz ^ NH
             kf += 1.0f;
-            if (((k + 1 + rot) & 15) == 0) kf -= 16.0f;
+            if (((k + 1 + rot) & (NH - 1)) == 0) kf -= (float)NH;
             const float2 dep = __ffma2_rn(kf2, dW2, W02);
             const float2 rw = make_float2(dc::rcp_approx(dep.x), dc::rcp_approx(dep.y));
             const float2 u = __ffma2_rn(__ffma2_rn(kf2, dU2, U02), rw, cul2);
@@ -375,8 +378,11 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
               i10[0] = __float2int_rn(g10.x), i10[1] = __float2int_rn(g10.y);
               i11[0] = __float2int_rn(g11.x), i11[1] = __float2int_rn(g11.y);
             }
-            red_add4(__float_as_uint(ad.x), i00[0], i01[0], i10[0], i11[0]);
-            red_add4(__float_as_uint(ad.y), i00[1], i01[1], i10[1], i11[1]);
+            // a masked voxel's zeros would only take atomics (and collide)
+            if (gv[k].x != 0.0f)
+              red_add4(__float_as_uint(ad.x), i00[0], i01[0], i10[0], i11[0]);
+            if (gv[k].y != 0.0f)
+              red_add4(__float_as_uint(ad.y), i00[1], i01[1], i10[1], i11[1]);
           }
         };
         if (any) {
@@ -394,10 +400,10 @@ __global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, 
         cur ^= 1;
       } else if (any) {
 #pragma unroll
-        for (int k = 0; k < TB_NZ; ++k) {
-          const float gk = (k & 16) ? gv[k & 15].y : gv[k & 15].x;
+        for (int k = 0; k < NZ; ++k) {
+          const float gk = (k & NH) ? gv[k & (NH - 1)].y : gv[k & (NH - 1)].x;
           if (gk == 0.0f) continue;
-          const float kf = (float)((((k & 15) + rot) & 15) + (off ^ (k & 16)));
+          const float kf = (float)((((k & (NH - 1)) + rot) & (NH - 1)) + (off ^ (k & NH)));
           float dep = fmaf(kf, dW, W0);
           if (!(dep > 0.0f)) continue;
           float rw = __frcp_rn(dep);
@@ -461,8 +467,11 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
   if (getenv("DC_BP_ADJ_GLOBAL")) {
     k_bp3d_adj<<<grid, blk, 0, st>>>(a);
   } else {
+    // 16-deep boxes where 32-deep ones mostly do not fit the tile (and would
+    // scatter into global memory): bp_plan's judgement
+    const int nz = g->bp_fit32 ? 32 : 16;
     dim3 gridt((d.vol_x + TB_TX - 1) / TB_TX, (d.vol_y + TB_TY - 1) / TB_TY,
-               ((d.vol_z + TB_NZ - 1) / TB_NZ) * B);
+               ((d.vol_z + nz - 1) / nz) * B);
     // few boxes share their views among CTAs (a view's gradient is summed by
     // atomics anyway), up to the three CTAs that an SM holds and down to 8
     // views each
@@ -471,10 +480,10 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
     while (split < 16 && 2 * split * boxes <= 456 && d.n_views >= 16 * split) split *= 2;
     gridt.z *= split;
     // float4 atomics need 16-byte pixel quads
-    if ((a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0)
-      k_bp3d_adj_tile<true><<<gridt, blk, 0, st>>>(a, split);
-    else
-      k_bp3d_adj_tile<false><<<gridt, blk, 0, st>>>(a, split);
+    const bool vec = (a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0;
+    auto kernel = nz == 32 ? (vec ? k_bp3d_adj_tile<true, 32> : k_bp3d_adj_tile<false, 32>)
+                           : (vec ? k_bp3d_adj_tile<true, 16> : k_bp3d_adj_tile<false, 16>);
+    kernel<<<gridt, blk, 0, st>>>(a, split);
   }
   DC_CHECK_LAUNCH("k_bp3d_adj");
   return DC_OK;
