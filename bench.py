@@ -96,7 +96,7 @@ def parse():
     ap.add_argument("--profile-case", choices=["filter_bp", "adj"], default=None,
                     help="run one small case twice for an ncu capture and exit: filter_bp = "
                          "the headline orbit, detector and planes with a 256^3 volume at the "
-                         "headline voxel size (19 images per filter chunk); adj = the "
+                         "headline voxel size (20 images per filter chunk); adj = the "
                          "backprojection transpose on the 256^3 sinusoid training geometry "
                          "with 90 views, batch 1")
     return ap.parse_args()
@@ -112,7 +112,7 @@ def profile_case(case: str, dev, storage: str = "f32"):
         desc = w.desc_dict()
         desc.update(vol_x=256, vol_y=256, vol_z=256)
         geom = api.Geometry(desc, w.matrices(), w.orbit.vdl)
-        api.dc_geometry_set_tuning(geom, 19, 32)
+        api.dc_geometry_set_tuning(geom, 20, 32)
         g = torch.randn((1, w.n_views, w.det_rows, w.det_cols), device=dev)
         for _ in range(2):
             gF, _ = api.dc_filter(geom, g, None, storage)
@@ -193,9 +193,9 @@ def load_peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0}, "fallback"
 
 
-KERNEL_SOURCES = {"k_bp3d": "paper_2410_14900_gb300/csrc/dc_backproject.cu",
-                  "k_linesum": "paper_2410_14900_gb300/csrc/dc_filter.cu",
-                  "k_bp2d": "paper_2410_14900_gb300/csrc/dc_filter.cu"}
+KERNEL_SOURCES = {"k_bp3d": "paper_2410_14900_gb300/csrc/dc_bp_box.cuh",
+                  "k_linesum": "paper_2410_14900_gb300/csrc/dc_filter_quad.cuh",
+                  "k_bp2d": "paper_2410_14900_gb300/csrc/dc_filter_quad.cuh"}
 
 
 def recorded_traffic(kernel: str, per_launch_units: float):
@@ -559,7 +559,7 @@ def paper_shape_measure(args, dev, L):
     w = synth.workload("paper400")
     geom = api.Geometry(w.desc_dict(), w.matrices(), w.orbit.vdl)
     st = args.storage if args.storage in ("f32", "f32x2") else "f32"
-    tuned = tune.autotune(geom, st, chunks=(8, 12, 16, 20, 25), nzs=(16, 32))
+    tuned = tune.autotune(geom, st, chunks=(24, 48, 64, 96, 128), nzs=(16, 32))
     g = synth.project_phantom(w.phantoms()[0], w.orbit, w.det_rows, w.det_cols, w.pitch,
                               device=dev, dtype=torch.float32)[None].contiguous()
     gF = torch.empty(api.gF_shape(geom, 1, st), device=dev)
@@ -617,7 +617,7 @@ def run_ours(args, rank, world, local_rank):
     geom = api.Geometry(desc, w.matrices(), w.orbit.vdl)
     # tile and chunk sizes picked by the autotuner (cached per problem shape)
     from paper_2410_14900_gb300 import tune
-    tuned = tune.autotune(geom, args.storage, chunks=(8, 12, 16, 19, 24), nzs=(16, 32))
+    tuned = tune.autotune(geom, args.storage, chunks=(24, 48, 64, 84, 128), nzs=(16, 32))
     # every rank reconstructs its own seeded phantom (independent problems)
     from paper_2410_14900_gb300 import sharding
     blobs = synth.random_ellipsoids(np.random.default_rng(sharding.rank_seed(w.seed, rank)),

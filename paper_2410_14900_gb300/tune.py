@@ -26,8 +26,9 @@ def cache_path() -> str:
 
 def shape_key(geom: api.Geometry, dtype: str = "f32") -> str:
     d = geom.desc
+    # q4: timed with the four-image filter kernels, which want larger chunks
     return "V{n_views}_H{det_rows}_W{det_cols}_mu{n_mu}_s{n_s}_vol{vol_z}x{vol_y}x{vol_x}".format(
-        **d) + f"_{dtype}"
+        **d) + f"_{dtype}_q4"
 
 
 def _load():
@@ -61,7 +62,7 @@ def _time(fn, reps=2):
 
 
 def autotune(geom: api.Geometry, dtype: str = "f32", use_cache: bool = True,
-             chunks=(8, 16, 32), nzs=(16, 32), kahan: bool = False) -> dict:
+             chunks=(16, 32, 64, 128, 256), nzs=(16, 32), kahan: bool = False) -> dict:
     """Pick chunk_images and bp_nz for `geom`, apply them and return them
     (the backprojection timed with Kahan summation when `kahan`)."""
     key = shape_key(geom, dtype) + ("|kahan" if kahan else "")
