@@ -161,10 +161,7 @@ void free_geometry(dc_geometry *g) {
   cudaFree(g->mu_order);
   cudaFree(g->groups);
   cudaFree(g->q_groups);
-  cudaFree(g->w_imgT);
-  cudaFree(g->w_img);
-  cudaFree(g->w_sinoA);
-  cudaFree(g->w_sinoB);
+  cudaFree(g->w_img);  // with w_imgT, w_sinoA and w_sinoB
   cudaFree(g->w_absmax);
   cudaFree(g->w_flags);
   if (g->aux_ready) {
