@@ -298,9 +298,9 @@ int dc_gauss_smooth(int V, int n_mu, int n_s, float sigma, int radius, int adjoi
  * (chunked launches, recorded in the same graph); with
  * DC_PERSISTENT_FILTER it is one persistent launch whose CTAs (one per SM)
  * take (problem, view) images from a device counter, largest per-image
- * work first, so the whole run is two persistent launches.  (On GB300 that
- * kernel runs its 2-D backprojection at half the warps per SM of the
- * chunked kernel and is ~11% slower; it is kept for launch-bound uses.)
+ * work first, so the whole run is two persistent launches.  (That kernel
+ * takes one image at a time where the chunked kernels take four: twelve
+ * uneven orbits need 792 ms with it and 475 ms without on a GB300.)
  * With the flag, problems whose detector or sinogram rows do not fit that
  * kernel's shared memory fall back to the per-problem calls, and so does
  * every problem of a DC_F32X2 batch (the pairs are made by the chunked

@@ -5,7 +5,8 @@
 //   g^F = w_d A2d^T D_b (W K) S                 (shift-variant filter, Eq. 11)
 //
 // and its reverse mode.  Views are processed in chunks of images (view x
-// batch item) so that the work area stays in L2:
+// batch item); where every view has the same principal point an image set is
+// four images interleaved (dc_filter_quad.cuh), otherwise one:
 //
 //   k_prep      weight (w_cos or w_d) and write the image with padded rows
 //   k_linesum   Joseph line sums of every (mu, s) line of an image, streamed
@@ -14,8 +15,7 @@
 //               the band step as the fastest index; neighbouring lines of a
 //               warp take the s-difference by shuffle so that D_f never
 //               subtracts two large sums; the epilogue applies w_sino, K, W
-//               and D_b (or the adjoint chain); four images at once where
-//               every view has the same principal point (k_linesum4)
+//               and D_b (or the adjoint chain)
 //   k_bp2d      pixel-driven A2d^T: each pixel gathers the two sinogram taps
 //               of every angle (the exact transpose of the Joseph weights),
 //               angles streamed through shared memory with bulk copies; the
