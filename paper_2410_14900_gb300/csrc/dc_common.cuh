@@ -164,9 +164,10 @@ struct dc_geometry {
   float *w_imgT;             // [chunk / 4][W][H][4] (w_img holds [chunk / 4][H][W][4])
   CUtensorMap q_tm_cols, q_tm_rows;  // over w_imgT and w_img
   // quad sinograms (w_sinoA, w_sinoB as [chunk / 4][n_mu][NSp][4]): the
-  // s-windows of the 2-D backprojection's tiles of q_ry rows per thread
+  // s-windows of the 2-D backprojection's tiles of q_ry rows per thread, q_nwx
+  // warps side by side
   CUtensorMap q_tm_sinoA, q_tm_sinoB;
-  int q_ry;
+  int q_ry, q_nwx;
   float *w_img;              // [chunk][H][Wp]
   float *w_sinoA;            // [chunk][n_mu][NSp]
   float *w_sinoB;            // [chunk][n_mu][NSp]

@@ -926,7 +926,7 @@ bool multi_tap(const dc_geometry *g) { return g->d.ds < g->d.pitch * (1.0 - 1e-1
 template <int NT, int RY>
 int launch_bp2d4_t(const dc_geometry *g, BP2Args &a, const B4Shape &sh, const CUtensorMap &tm,
                    cudaStream_t st) {
-  const size_t sm = (size_t)2 * B4_MC * sh.lwb * sh.nb * 16;
+  const size_t sm = b4_smem(sh);
   DC_CUDA(cudaFuncSetAttribute(k_bp2d4<NT, RY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)sm));
   const int tx = 32 * sh.nwx, ty = RY * (8 / sh.nwx);
@@ -938,7 +938,7 @@ int launch_bp2d4_t(const dc_geometry *g, BP2Args &a, const B4Shape &sh, const CU
 
 template <int NT>
 int launch_bp2d4(const dc_geometry *g, BP2Args &a, cudaStream_t st) {
-  const B4Shape sh = b4_shape(a.H, a.W, g->d.pitch, g->d.ds, g->q_ry);
+  const B4Shape sh = b4_arrange(g->q_nwx, g->d.pitch, g->d.ds, g->q_ry);
   const CUtensorMap &tm = (a.sino == g->w_sinoB) ? g->q_tm_sinoB : g->q_tm_sinoA;
   return g->q_ry == 2 ? launch_bp2d4_t<NT, 2>(g, a, sh, tm, st)
                       : launch_bp2d4_t<NT, 8>(g, a, sh, tm, st);
@@ -1340,8 +1340,11 @@ int alloc_workspace(dc_geometry *g) {
   }
   if (g->quad) {
     const size_t ng = ci / 4, n0 = 4 * (size_t)g->NSp, n1 = d.n_mu;
-    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, std::min(d.n_views, ci));
-    const int lwb = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry).lwb;
+    const int images = std::min(d.n_views, ci);
+    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, images);
+    const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, images);
+    g->q_nwx = b4.nwx;
+    const int lwb = b4.lwb;
     if (!encode_map_f32(&g->q_tm_sinoA, g->w_sinoA, n0, n1, ng, 4 * lwb, 1) ||
         !encode_map_f32(&g->q_tm_sinoB, g->w_sinoB, n0, n1, ng, 4 * lwb, 1))
       g->quad = 0;

@@ -543,6 +543,9 @@ struct B4Mu {
   unsigned pad0, pad1;
 };
 
+// two stages of a tile's window
+inline size_t b4_smem(const B4Shape &s) { return (size_t)2 * B4_MC * s.lwb * s.nb * 16; }
+
 // taps per pixel and angle: the hat's half-width is at most pitch / ds bins
 template <int NT>
 constexpr int b4_left() { return NT / 2 - 1; }
@@ -551,26 +554,58 @@ inline int b4_taps(double pitch, double ds) {
   return ds >= pitch * (1.0 - 1e-12) ? 2 : 2.0 * ds >= pitch * (1.0 - 1e-12) ? 4 : 6;
 }
 
-// the warps' arrangement with the fewest pixels outside the detector (the
-// squarest of equals: the smallest window), and the window of its tile
-inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY) {
+// Dynamic shared memory up to which two CTAs share an SM (228 KB, 1 KB of it
+// the system's per CTA, beside 2 KB of static tables), and the most that any
+// launch asks for, whatever its geometry.
+constexpr int B4_SMEM_TWO = 111 * 1024;
+constexpr int B4_SMEM_MAX = 224 * 1024;
+
+// the arrangement of nwx warps side by side and the window of its tile
+inline B4Shape b4_arrange(int nwx, double pitch, double ds, int RY) {
   B4Shape s;
-  long best = 0;
-  const int order[4] = {2, 1, 4, 8};
-  for (int i = 0; i < 4; ++i) {
-    const int tx = 32 * order[i], ty = RY * (8 / order[i]);
-    const long px = (long)((W + tx - 1) / tx) * tx * ((H + ty - 1) / ty) * ty;
-    if (i == 0 || px < best) {
-      best = px;
-      s.nwx = order[i];
-    }
-  }
-  const int tx = 32 * s.nwx, ty = RY * (8 / s.nwx), nt = b4_taps(pitch, ds);
+  s.nwx = nwx;
+  const int tx = 32 * nwx, ty = RY * (8 / nwx), nt = b4_taps(pitch, ds);
   const double span = std::sqrt((tx - 1.0) * (tx - 1.0) + (ty - 1.0) * (ty - 1.0)) * pitch / ds;
   const int need = (int)(span + 0.1) + 3 + nt;
   s.nb = (need + 63) / 64;
   s.lwb = (((need + s.nb - 1) / s.nb) + 7) & ~7;
   return s;
+}
+
+inline long b4_tiles(int H, int W, const B4Shape &s, int RY, int images) {
+  const int tx = 32 * s.nwx, ty = RY * (8 / s.nwx);
+  return (long)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * ((images + 3) / 4);
+}
+
+// The warps' arrangement with the least time for `images` images among those
+// whose stages an SM holds (the squarest of equals: the smallest window).  At
+// ds >= pitch / 3 the squarest one always fits (112 KB); 256 x 8 tiles want 140
+// KB at ds = pitch, 288 at pitch / 2.  With 8 rows per thread that time is what
+// an SM's share of the tiles takes: two CTAs together 2 units, one alone, or at
+// a time because two do not fit, 1.28 (two taps) or 1.13 (more): 96 images,
+// 180 angles, ds = pitch: 360 x 512 974 us in 15 rounds of 256 x 8 tiles, one
+// CTA per SM, 775 in 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds
+// of 256 x 8, 655 in 5 of 128 x 16.  With 2 rows (grids of less than a wave) it
+// is the pixels computed, those outside the detector too.
+inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int images) {
+  const double alone = b4_taps(pitch, ds) == 2 ? 1.28 : 1.13;
+  B4Shape best = {};
+  double least = -1.0;
+  const int order[4] = {2, 1, 4, 8};
+  for (int i = 0; i < 4; ++i) {
+    const B4Shape s = b4_arrange(order[i], pitch, ds, RY);
+    const size_t sm = b4_smem(s);
+    if (i > 0 && sm > (size_t)B4_SMEM_MAX) continue;
+    const long tiles = b4_tiles(H, W, s, RY, images), n = (tiles + 151) / 152;
+    const double cost = RY == 2 ? (double)tiles
+                        : sm <= (size_t)B4_SMEM_TWO ? 2.0 * (n / 2) + alone * (n % 2)
+                                                    : alone * n;
+    if (least < 0.0 || cost < least) {
+      least = cost;
+      best = s;
+    }
+  }
+  return best;
 }
 
 // Rows per thread: 8, unless the 2048-pixel tiles of the views at hand leave
@@ -579,10 +614,7 @@ inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY) {
 // geometry, so that an image's result does not depend on the chunk or batch
 // that it comes in.
 inline int b4_rows(int H, int W, double pitch, double ds, int images) {
-  const B4Shape s = b4_shape(H, W, pitch, ds, 8);
-  const int tx = 32 * s.nwx, ty = 64 / s.nwx;
-  const long tiles = (long)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * ((images + 3) / 4);
-  return tiles < 152 ? 2 : 8;
+  return b4_tiles(H, W, b4_shape(H, W, pitch, ds, 8, images), 8, images) < 152 ? 2 : 8;
 }
 
 // 8 rows per thread want the registers of two CTAs per SM (496 images of 384 x
