@@ -927,8 +927,10 @@ template <int NT, int RY>
 int launch_bp2d4_t(const dc_geometry *g, BP2Args &a, const B4Shape &sh, const CUtensorMap &tm,
                    cudaStream_t st) {
   const size_t sm = b4_smem(sh);
+  // the limit belongs to the kernel, not to the launch: one value for all
+  // geometries, so that no thread lowers it under another's launch
   DC_CUDA(cudaFuncSetAttribute(k_bp2d4<NT, RY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sm));
+                               B4_SMEM_MAX));
   const int tx = 32 * sh.nwx, ty = RY * (8 / sh.nwx);
   dim3 grid((a.W + tx - 1) / tx, (a.H + ty - 1) / ty, (a.n_img + 3) / 4);
   k_bp2d4<NT, RY><<<grid, B4_THREADS, sm, st>>>(a, sh, tm);
