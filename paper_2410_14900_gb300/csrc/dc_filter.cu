@@ -1515,8 +1515,10 @@ int batch_filter_create(int n, dc_geometry *const *geoms, int dtype, void *const
     batch_filter_destroy(p);
     return fail(DC_ERR_UNSUPPORTED, "batched filter: sinogram rows too long for its shared memory");
   }
+  // the limit belongs to the kernel: one value for all plans, so that none
+  // lowers it under another's launch
   cudaError_t e = cudaFuncSetAttribute(k_filter_batched, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)p->smem);
+                                       (int)budget);
   int per_sm = 0, sms = 0;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_filter_batched, BF_THREADS, p->smem);

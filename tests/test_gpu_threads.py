@@ -3,7 +3,6 @@ thread and a stream of its own, and batches that outlive the creation of
 others: the shared-memory limit of a kernel belongs to the process."""
 import threading
 
-import numpy as np
 import pytest
 import torch
 
@@ -49,3 +48,17 @@ def test_two_threads_with_their_own_handles():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_a_batch_runs_after_a_smaller_one_was_created():
+    big, small = _geometry(5, 120, 700, 900), _geometry(5, 16, 16, 16)
+    g = torch.rand((5, 120, 700), device="cuda")
+    vol, ref = torch.empty(big.vol_shape, device="cuda"), torch.empty(big.vol_shape, device="cuda")
+    first = api.Batch([big], persistent_filter=True)
+    first.run([g], [ref])
+    second = api.Batch([small], persistent_filter=True)
+    first.run([g], [vol])
+    torch.cuda.synchronize()
+    assert torch.equal(vol, ref)
+    second.close()
+    first.close()
