@@ -330,23 +330,45 @@ int backproject_check(const dc_geometry *g, int B, const void *gF, int dtype,
 int backproject_slab(const dc_geometry *g, int B, const void *gF, int dtype,
                      const float *gF_scale, float *vol, unsigned flags, int z_begin, int z_end,
                      cudaStream_t st, bool *used) {
-  BPArgs a = bp_args(g, B, gF, dtype, gF_scale, vol, flags);
-  a.z_begin = z_begin;
-  a.z_end = z_end;
-  const bool kahan = (flags & DC_KAHAN) != 0;
   *used = false;
   if (getenv("DC_BP_NO_TMA")) return DC_OK;
-  ProfScope ps(KID_BP3D, st);
-  int rc;
-  switch (dtype) {
-    case DC_F32: rc = launch_bp_tma<float>(g, a, dtype, kahan, st, used); break;
-    case DC_F32X2: rc = launch_bp_tma<float2>(g, a, dtype, kahan, st, used); break;
-    case DC_BF16: rc = launch_bp_tma<__nv_bfloat16>(g, a, dtype, kahan, st, used); break;
-    default: rc = launch_bp_tma<__half>(g, a, dtype, kahan, st, used); break;
+  // A launch takes at most 65535 CTAs along z: layers of boxes times batch
+  // items times the CTAs that share a box's views.  More go in several
+  // launches, whole items each (a result does not depend on where they part).
+  const dc_geometry_desc &d = g->d;
+  const int nz = g->bp_nz, share = nz == 16 ? g->bp_split : 1, most = 65535 / share;
+  const int layers = bp_layers(z_begin, z_end, nz);
+  if (layers > most) {
+    const int zm = z_begin + most * nz;
+    int rc = backproject_slab(g, B, gF, dtype, gF_scale, vol, flags, z_begin, zm, st, used);
+    if (rc || !*used) return rc;
+    return backproject_slab(g, B, gF, dtype, gF_scale, vol, flags, zm, z_end, st, used);
   }
-  if (rc) return rc;
-  if (*used) DC_CHECK_LAUNCH("k_bp3d_tma");
-  else return backproject_rows(g, B, gF, dtype, gF_scale, vol, flags, z_begin, z_end, st, used);
+  const size_t item = (size_t)d.n_views * d.det_rows * d.det_cols * pixel_bytes(dtype);
+  const size_t nvox = (size_t)d.vol_x * d.vol_y * d.vol_z;
+  const int per = std::min(B, most / layers);
+  for (int b = 0; b < B; b += per) {
+    const int n = std::min(per, B - b);
+    const void *p = (const char *)gF + b * item;
+    const float *sc = gF_scale ? gF_scale + (size_t)b * d.n_views : nullptr;
+    float *v = vol + b * nvox;
+    BPArgs a = bp_args(g, n, p, dtype, sc, v, flags);
+    a.z_begin = z_begin;
+    a.z_end = z_end;
+    const bool kahan = (flags & DC_KAHAN) != 0;
+    ProfScope ps(KID_BP3D, st);
+    int rc;
+    switch (dtype) {
+      case DC_F32: rc = launch_bp_tma<float>(g, a, dtype, kahan, st, used); break;
+      case DC_F32X2: rc = launch_bp_tma<float2>(g, a, dtype, kahan, st, used); break;
+      case DC_BF16: rc = launch_bp_tma<__nv_bfloat16>(g, a, dtype, kahan, st, used); break;
+      default: rc = launch_bp_tma<__half>(g, a, dtype, kahan, st, used); break;
+    }
+    if (rc) return rc;
+    if (*used) DC_CHECK_LAUNCH("k_bp3d_tma");
+    else if ((rc = backproject_rows(g, n, p, dtype, sc, v, flags, z_begin, z_end, st, used))) return rc;
+    if (!*used) return DC_OK;  // the layout that neither reads: true of every item
+  }
   return DC_OK;
 }
 

@@ -1,5 +1,6 @@
 // dc_backproject_adj.cu -- the transpose of the voxel-driven cone-beam
 // backprojection (Ye et al., DRACO, Sec. 2.3: the reverse mode of Eq. 5).
+#include <algorithm>
 #include <cstdlib>
 #include <string>
 
@@ -469,21 +470,32 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
   } else {
     // 16-deep boxes where 32-deep ones mostly do not fit the tile (and would
     // scatter into global memory): bp_plan's judgement
-    const int nz = g->bp_fit32 ? 32 : 16;
-    dim3 gridt((d.vol_x + TB_TX - 1) / TB_TX, (d.vol_y + TB_TY - 1) / TB_TY,
-               ((d.vol_z + nz - 1) / nz) * B);
+    const int nz = g->bp_fit32 || d.vol_z > 16 * 65535 ? 32 : 16;
+    const int layers = (d.vol_z + nz - 1) / nz;
+    dim3 gridt((d.vol_x + TB_TX - 1) / TB_TX, (d.vol_y + TB_TY - 1) / TB_TY);
     // few boxes share their views among CTAs (a view's gradient is summed by
     // atomics anyway), up to the three CTAs that an SM holds and down to 8
     // views each
-    const long boxes = (long)gridt.x * gridt.y * gridt.z;
+    const long boxes = (long)gridt.x * gridt.y * layers * B;
     int split = 1;
     while (split < 16 && 2 * split * boxes <= 456 && d.n_views >= 16 * split) split *= 2;
-    gridt.z *= split;
     // float4 atomics need 16-byte pixel quads
     const bool vec = (a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0;
     auto kernel = nz == 32 ? (vec ? k_bp3d_adj_tile<true, 32> : k_bp3d_adj_tile<false, 32>)
                            : (vec ? k_bp3d_adj_tile<true, 16> : k_bp3d_adj_tile<false, 16>);
-    kernel<<<gridt, blk, 0, st>>>(a, split);
+    // whole items per launch, at most 65535 CTAs along z
+    const int per = std::min(B, std::max(1, 65535 / (layers * split)));
+    const size_t np = (size_t)d.n_views * d.det_rows * d.det_cols,
+                 nvox = (size_t)d.vol_x * d.vol_y * d.vol_z;
+    for (int b = 0; b < B; b += per) {
+      BPAdjArgs c = a;
+      c.grad_vol += b * nvox;
+      if (c.relu_vol) c.relu_vol += b * nvox;
+      c.grad_gF += b * np;
+      c.B = std::min(per, B - b);
+      gridt.z = layers * c.B * split;
+      kernel<<<gridt, blk, 0, st>>>(c, split);
+    }
   }
   DC_CHECK_LAUNCH("k_bp3d_adj");
   return DC_OK;
