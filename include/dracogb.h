@@ -73,7 +73,10 @@ extern "C" {
 
 /* dc_backproject flags */
 #define DC_ACCUM 1u           /* add into vol instead of overwriting        */
-#define DC_KAHAN 2u           /* compensated (Kahan) summation over views   */
+/* Compensated (Kahan) summation over views: of the sums over 32 views each,
+ * plain FP32 inside, where rows of g^F are multiples of 16 bytes from an
+ * aligned base; of every view's term otherwise. */
+#define DC_KAHAN 2u
 #define DC_RELU 4u            /* ReLU after the sum over views (Sec. 2.3)   */
 /* dc_batch_create flag: filter every problem in one persistent launch */
 #define DC_PERSISTENT_FILTER 8u

@@ -6,7 +6,7 @@
 //
 // 128 x 512 x 512 voxels from 400 views of 480 x 620 BF16 pixels (rows of 1240
 // bytes) with compensated sums: 36.1 ms by bounds-checked gathers from global
-// memory (k_bp3d), 13.4 ms here.
+// memory (k_bp3d), 13.8 ms here.
 #include "dc_bp_box.cuh"
 
 namespace {

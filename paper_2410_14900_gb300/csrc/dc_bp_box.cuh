@@ -237,24 +237,47 @@ __device__ __forceinline__ bool bp_box(const BPArgs &a, float *vol, const CUtens
   // every view: the FP32 error is that of a TB_VCH-term sum, at 1/TB_VCH of
   // the per-view compensation cost.  The total and its compensation are
   // touched once per chunk, in a rolled loop, and so live in local memory
-  // (in registers beside the chunk sum they cost a quarter of the time:
-  // 16.3 against 13.4 ms for 128 x 512 x 512 voxels and 400 views of BF16
-  // rows).  Without KAHAN terms go to acc2.
+  // (in registers beside the chunk sum they cost a quarter of the time).
+  // Footprints staged by rows (LD != LD_TMA) compensate every view's term, as
+  // the kernel for such rows always did; neg2 is the negative of the running
+  // compensation (13.8 ms for 128 x 512 x 512 voxels and 400 views of BF16
+  // rows, 13.4 with chunk sums).  Without KAHAN terms go to acc2.
+  constexpr bool PER_VIEW = KAHAN && LD != LD_TMA, CHUNKED = KAHAN && !PER_VIEW;
   constexpr int NH = NZ / 2;
-  float2 acc2[NH];
-  float tot[KAHAN ? NZ : 1], cmp[KAHAN ? NZ : 1], prt[KAHAN ? NZ : 1];
+  float2 acc2[NH], neg2[PER_VIEW ? NH : 1];
+  float tot[CHUNKED ? NZ : 1], cmp[CHUNKED ? NZ : 1], prt[CHUNKED ? NZ : 1];
 #pragma unroll
   for (int h = 0; h < NH; ++h) acc2[h] = make_float2(0.0f, 0.0f);
-  if (KAHAN) {
+  if constexpr (PER_VIEW) {
+#pragma unroll
+    for (int h = 0; h < NH; ++h) neg2[h] = make_float2(0.0f, 0.0f);
+  }
+  if (CHUNKED) {
 #pragma unroll 1
     for (int k = 0; k < NZ; ++k) tot[k] = cmp[k] = 0.0f;
   }
   // a pair of terms val * wt into voxels (h, h + NH); one term into voxel k
-  auto add2 = [&](int h, float2 val, float2 wt) { acc2[h] = __ffma2_rn(val, wt, acc2[h]); };
+  auto add2 = [&](int h, float2 val, float2 wt) {
+    if constexpr (PER_VIEW) {
+      const float2 m1 = make_float2(-1.0f, -1.0f);
+      const float2 y = __ffma2_rn(val, wt, neg2[h]), t = __fadd2_rn(acc2[h], y);
+      neg2[h] = __ffma2_rn(__ffma2_rn(acc2[h], m1, t), m1, y);
+      acc2[h] = t;
+    } else {
+      acc2[h] = __ffma2_rn(val, wt, acc2[h]);
+    }
+  };
   auto add1 = [&](int k, float term) {
-    float2 &c = acc2[k < NH ? k : k - NH];
-    if (k < NH) c.x += term;
-    else c.y += term;
+    const int h = k < NH ? k : k - NH;
+    float &c = k < NH ? acc2[h].x : acc2[h].y;
+    if constexpr (PER_VIEW) {
+      float &n = k < NH ? neg2[h].x : neg2[h].y;
+      const float y = term + n, t = c + y;
+      n = y - (t - c);
+      c = t;
+    } else {
+      c += term;
+    }
   };
 
   bool ok = true;
@@ -554,7 +577,7 @@ __device__ __forceinline__ bool bp_box(const BPArgs &a, float *vol, const CUtens
         }
       }
     }
-    if (KAHAN && ok) {
+    if (CHUNKED && ok) {
 #pragma unroll
       for (int h = 0; h < NH; ++h) {
         prt[h] = acc2[h].x;
@@ -575,7 +598,7 @@ __device__ __forceinline__ bool bp_box(const BPArgs &a, float *vol, const CUtens
     __syncthreads();  // every thread is done with the stages
 #pragma unroll
     for (int k = 0; k < NZ; ++k)
-      part[k * (TB_TX * TB_TY) + tid] = KAHAN ? tot[k] : (k < NH) ? acc2[k].x : acc2[k - NH].y;
+      part[k * (TB_TX * TB_TY) + tid] = CHUNKED ? tot[k] : (k < NH) ? acc2[k].x : acc2[k - NH].y;
     return ok;
   }
   if (!ok) return false;
@@ -586,7 +609,7 @@ __device__ __forceinline__ bool bp_box(const BPArgs &a, float *vol, const CUtens
     const int iz = z0 + k;
     if (iz < z_own || iz >= a.z_end) continue;
     size_t o = (size_t)b * nvox + ((size_t)iz * a.ny + iy) * a.nx + ix;
-    float f = KAHAN ? tot[k] : (k < NH) ? acc2[k].x : acc2[k - NH].y;
+    float f = CHUNKED ? tot[k] : (k < NH) ? acc2[k].x : acc2[k - NH].y;
     if (a.flags & DC_ACCUM) f += vol[o];
     if ((a.flags & DC_RELU) && f < 0.0f) f = 0.0f;
     vol[o] = f;
