@@ -406,11 +406,26 @@ def transient_dtype(geom: Geometry, B: int, dtype: str = "f32") -> str:
     return "f32x2" if dtype == "f32" and B * geom.V * geom.H * geom.W >= 1 << 22 else dtype
 
 
+def with_transient(geom: Geometry, B: int, dtype: str, run):
+    """run(storage form of the transient g^F); in the caller's own form where
+    the pairs, twice its memory, do not fit."""
+    form = transient_dtype(geom, B, dtype)
+    if form != dtype:
+        try:
+            return run(form)
+        except torch.cuda.OutOfMemoryError:
+            pass
+    return run(dtype)
+
+
 def reconstruct(geom: Geometry, g: torch.Tensor, W: Optional[torch.Tensor] = None,
                 dtype: str = "f32", kahan: bool = False, relu: bool = False) -> torch.Tensor:
     """Eq. 12: f = A3d^T w_d A2d^T D w_red w_sino D A2d w_cos g."""
-    gF, sc = dc_filter(geom, g, W, transient_dtype(geom, g.shape[0], dtype))
-    return dc_backproject(geom, gF, sc, kahan=kahan, relu=relu)
+    def run(form):
+        gF, sc = dc_filter(geom, g, W, form)
+        return dc_backproject(geom, gF, sc, kahan=kahan, relu=relu)
+
+    return with_transient(geom, g.shape[0], dtype, run)
 
 
 def dc_reconstruct_host(geom: Geometry, g_host: torch.Tensor, vol_host: torch.Tensor,

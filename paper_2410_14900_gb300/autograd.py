@@ -39,9 +39,12 @@ class DefriseClackFunction(torch.autograd.Function):
         if cache_s and need_grad:
             S = torch.empty((g.shape[0], geom.V) + geom.sino_shape, device=g.device,
                             dtype=torch.float32)
-        gF, _ = api.dc_filter(geom, g, Wc, api.transient_dtype(geom, g.shape[0]), S_out=S)
-        vol = api.dc_backproject(geom, gF, relu=relu)
-        del gF
+
+        def run(form):
+            gF, _ = api.dc_filter(geom, g, Wc, form, S_out=S)
+            return api.dc_backproject(geom, gF, relu=relu)
+
+        vol = api.with_transient(geom, g.shape[0], "f32", run)
         ctx.geom = geom
         ctx.relu = relu
         ctx.view_chunk = view_chunk

@@ -1,0 +1,41 @@
+"""The storage form of a g^F that only the next backprojection reads: what
+happens where FP32 pairs, twice the memory, do not fit."""
+import pytest
+import torch
+
+from paper_2410_14900_gb300 import api, synth
+from paper_2410_14900_gb300.autograd import reconstruct
+
+pytestmark = pytest.mark.gpu
+
+
+def _geometry(V, H, W, n, voxel):
+    o = synth.sinusoid_orbit(V)
+    desc = dict(n_views=V, det_rows=H, det_cols=W, n_mu=8, n_s=64, pitch=1.0, ds=4.0, vol_x=n,
+                vol_y=n, vol_z=n, voxel=(voxel,) * 3, vol_center=(1.0, 2.0, -1.0), closed_orbit=1)
+    return api.Geometry(desc, synth.projection_matrices(o, H, W, 1.0), o.vdl)
+
+
+def test_pairs_that_do_not_fit_give_way():
+    V, H, W, n = 160, 256, 256, 160
+    geom = _geometry(V, H, W, n, 0.9)
+    assert api.transient_dtype(geom, 1) == "f32x2"
+    g = torch.rand((1, V, H, W), device="cuda")
+    gF, _ = api.dc_filter(geom, g, None, "f32")
+    ref = api.dc_backproject(geom, gF)
+    del gF
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # room for g^F in FP32 (42 MB) and the volume (16 MB), not for the pairs (84 MB)
+    room = torch.cuda.memory_reserved() + (72 << 20)
+    total = torch.cuda.get_device_properties(0).total_memory
+    torch.cuda.set_per_process_memory_fraction(room / total)
+    try:
+        vol = api.reconstruct(geom, g)
+        same = torch.equal(vol, ref)
+        del vol
+        torch.cuda.empty_cache()
+        net = reconstruct(g, None, geom)
+        assert same and torch.equal(net, ref)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
