@@ -86,6 +86,16 @@ class Geometry:
         check(rc, "dc_setup_geometry")
         self._h = h
         self._lib = L
+        self._px_per_mm = None
+
+    def pixels_per_mm(self) -> float:
+        """Detector pixels per mm at the volume's centre, in the middle view."""
+        if self._px_per_mm is None:
+            v = dc_get_view_geometry(self)[self.V // 2].tolist()
+            c = self.desc.get("vol_center", (0.0, 0.0, 0.0))
+            depth = sum((v[t] - c[t]) * v[9 + t] for t in range(3))
+            self._px_per_mm = v[12] / (depth * self.desc["pitch"])
+        return self._px_per_mm
 
     @property
     def handle(self):
@@ -400,10 +410,23 @@ def transient_dtype(geom: Geometry, B: int, dtype: str = "f32") -> str:
     """Storage of a g^F that only the next backprojection reads.  FP32 goes
     through FP32 pairs (the same values, in the form that it interpolates from;
     twice the memory) where the staged boxes' conversions cost more than the
-    pass that writes the pairs: 360 views of 256 x 256 to 256^3 9.44 against
-    9.17 ms, 90 views of 128 x 128 x 2 items alike, 64 views of 64 x 64 109
-    against 111 us."""
-    return "f32x2" if dtype == "f32" and B * geom.V * geom.H * geom.W >= 1 << 22 else dtype
+    pass that writes the pairs: from 4M pixels (below, launches decide), where
+    the boxes' footprints fit their tiles and hold 6 values or more per pixel.
+    100 views of 256 x 256, sinusoid: at 1.6 pixels per voxel the pairs save 118
+    us of 192^3 voxels and 43 of 128^3, and cost 8 of 64^3; at 3 pixels per
+    voxel, where footprints do not fit, they cost 13 to 26."""
+    if dtype != "f32" or B * geom.V * geom.H * geom.W < 1 << 22 or geom.W % 2:
+        return dtype
+    d = geom.desc
+    nz = dc_geometry_get_tuning(geom)["bp_nz"]
+    px = geom.pixels_per_mm()
+    rows = (nz - 1) * d["voxel"][2] * px * 1.1 + 6
+    cols = 15 * (d["voxel"][0] ** 2 + d["voxel"][1] ** 2) ** 0.5 * px * 1.1 + 5
+    if rows > 48 or cols > 64:
+        return dtype
+    boxes = -(-d["vol_x"] // 16) * -(-d["vol_y"] // 16) * -(-d["vol_z"] // nz)
+    values = boxes * rows * (32 if cols <= 32 else 64)
+    return "f32x2" if values >= 6 * geom.H * geom.W else dtype
 
 
 def with_transient(geom: Geometry, B: int, dtype: str, run):

@@ -1,10 +1,13 @@
-"""The storage form of a g^F that only the next backprojection reads: what
-happens where FP32 pairs, twice the memory, do not fit."""
+"""The storage form of a g^F that only the next backprojection reads: which
+calls take FP32 pairs, that both forms agree, and what happens where the pairs,
+twice the memory, do not fit."""
 import pytest
 import torch
 
 from paper_2410_14900_gb300 import api, synth
 from paper_2410_14900_gb300.autograd import reconstruct
+
+from cases import rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -14,6 +17,28 @@ def _geometry(V, H, W, n, voxel):
     desc = dict(n_views=V, det_rows=H, det_cols=W, n_mu=8, n_s=64, pitch=1.0, ds=4.0, vol_x=n,
                 vol_y=n, vol_z=n, voxel=(voxel,) * 3, vol_center=(1.0, 2.0, -1.0), closed_orbit=1)
     return api.Geometry(desc, synth.projection_matrices(o, H, W, 1.0), o.vdl)
+
+
+# a volume of many boxes; one of few beside the same pixels; one pixel short of
+# 4M; voxels of three pixels, whose footprints do not fit a tile; odd rows
+@pytest.mark.parametrize("V,H,W,n,voxel,form", [
+    (64, 256, 256, 160, 0.9, "f32x2"), (64, 256, 256, 48, 0.9, "f32"),
+    (64, 256, 256, 16, 0.5, "f32"), (63, 256, 256, 160, 0.9, "f32"),
+    (64, 256, 256, 160, 1.9, "f32"), (66, 256, 255, 160, 0.9, "f32")])
+def test_form_and_agreement(V, H, W, n, voxel, form):
+    geom = _geometry(V, H, W, n, voxel)
+    assert api.transient_dtype(geom, 1) == form
+    for other in ("bf16", "f16", "f32x2"):
+        assert api.transient_dtype(geom, 1, other) == other
+    g = torch.rand((1, V, H, W), device="cuda")
+    gF, _ = api.dc_filter(geom, g, None, "f32")
+    ref = api.dc_backproject(geom, gF, relu=True)
+    vol = api.reconstruct(geom, g, relu=True)
+    net = reconstruct(g, None, geom, True)
+    assert torch.equal(vol, net)
+    if form == "f32":
+        assert torch.equal(vol, ref)
+    assert rel_l2(vol.double().cpu().numpy(), ref.double().cpu().numpy()) < 1e-5
 
 
 def test_pairs_that_do_not_fit_give_way():
