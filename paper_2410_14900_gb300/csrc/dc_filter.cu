@@ -1248,21 +1248,25 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 
 namespace dc {
 
-// Images that the work area holds.  The per-image kernels want a chunk that
-// stays in the 126 MB L2 (112 MB); the four-image kernels take few CTAs per
-// image, so larger chunks keep the last wave of a launch small (their L2
-// working set is the few images in flight).  The autotuner may use fewer
-// images per chunk.
-static int chunk_capacity(const dc_geometry *g) {
+constexpr long L2_MB = 112, QUAD_MB = 384;
+
+// Images that the work area holds, in `mb` MB of it: the per-image kernels
+// want a chunk that stays in the 126 MB L2 (112 MB); the four-image kernels take
+// few CTAs per image, so larger chunks keep the last wave of a launch small
+// (their L2 working set is the few images in flight): 384 MB, but no more images
+// than the views, or than the per-image kernels would take for several items.
+// The autotuner may use fewer images per chunk.
+static int chunk_capacity(const dc_geometry *g, bool quad, long mb) {
   const dc_geometry_desc &d = g->d;
   const size_t img = (size_t)d.det_rows * round4(d.det_cols), sino = (size_t)d.n_mu * round4(d.n_s);
-  const size_t per_img = ((g->quad ? 2 : 1) * img + 2 * sino) * sizeof(float);
-  const long target = (g->quad ? 384L : 112L) << 20;
+  const size_t per_img = ((quad ? 2 : 1) * img + 2 * sino) * sizeof(float);
   const char *env = getenv("DC_CHUNK_IMAGES");
-  int ci = env ? atoi(env) : (int)(target / (long)per_img);
-  if (ci < 4) ci = 4;
-  if (ci > 256) ci = 256;
-  return g->quad ? ci & ~3 : ci;
+  auto clamp = [](long n) { return std::min(std::max(n, 4L), 256L); };
+  auto quads = [](long n) { return (n + 3) & ~3L; };
+  if (env) return (int)(quad ? quads(clamp(atoi(env))) : clamp(atoi(env)));
+  const long most = clamp((mb << 20) / (long)per_img);
+  if (!quad) return (int)most;
+  return (int)std::min(most & ~3L, quads(std::max(d.n_views, chunk_capacity(g, false, L2_MB))));
 }
 
 // The four-image line sums share every sample position, so all views need
@@ -1286,9 +1290,7 @@ int quad_plan(dc_geometry *g) {
   const int nch = (d.n_s + 31) / 32, NSp = round4(d.n_s);
   const L4Shape sh = l4_shape(d.det_rows, d.det_cols);
   const int nb[2] = {(d.n_mu + 1) / 2, d.n_mu / 2};  // angles per branch, within one
-  g->quad = 1;
-  const int quads = (std::min(d.n_views, chunk_capacity(g)) + 3) / 4;
-  g->quad = 0;
+  const int quads = (std::min(d.n_views, chunk_capacity(g, true, QUAD_MB)) + 3) / 4;
   const double over = 23.2 * L4_RB / (d.det_rows + d.det_cols);
   double best = 0.0;
   for (int mg = 1; mg <= L4_MAX_MG && mg * nch <= L4_TASKS; ++mg) {
@@ -1316,23 +1318,38 @@ int alloc_workspace(dc_geometry *g) {
   g->NSp = round4(d.n_s);
   g->img_stride = (size_t)d.det_rows * g->Wp;
   g->sino_stride = (size_t)d.n_mu * g->NSp;
-  const int ci = chunk_capacity(g);
-  g->l2_images = std::max(4, (int)((112L << 20) /
-                                   (long)((g->img_stride + 2 * g->sino_stride) * sizeof(float))));
-  g->chunk_images = ci;
-  g->chunk_capacity = ci;
+  g->l2_images = chunk_capacity(g, false, L2_MB);
   bp_plan(g);
   g->ls_rb = linesum_band_rows(d.det_rows, d.det_cols, g->mg, g->NSp);
   if (g->ls_rb == 0 || bp2d_smem(g) > 200 * 1024)
     return fail(DC_ERR_UNSUPPORTED, "detector or sinogram rows too long for shared memory");
-  // one block (four allocations of this size cost 0.1 ms more), its parts on 1 KB
+  // one block (four allocations of this size cost 0.1 ms more), its parts on 1
+  // KB.  Where the four-image kernels' does not fit, a smaller one, and the
+  // per-image kernels' at the last.
   auto floats = [](size_t n) { return (n + 255) & ~(size_t)255; };
-  const size_t n_img = floats(g->img_stride * ci), n_sino = floats(g->sino_stride * ci);
-  const size_t n_imgT = g->quad ? floats((size_t)d.det_rows * d.det_cols * ci) : 0;
-  DC_CUDA(dmalloc((void **)&g->w_img, sizeof(float) * (n_img + n_imgT + 2 * n_sino)));
-  g->w_imgT = g->quad ? g->w_img + n_img : nullptr;
-  g->w_sinoA = g->w_img + n_img + n_imgT;
-  g->w_sinoB = g->w_sinoA + n_sino;
+  const struct {
+    bool quad;
+    long mb;
+  } tries[3] = {{true, QUAD_MB}, {true, L2_MB}, {false, L2_MB}};
+  int ci = 0;
+  cudaError_t e = cudaErrorMemoryAllocation;
+  for (int t = g->quad ? 0 : 2; t < 3 && e == cudaErrorMemoryAllocation; ++t) {
+    g->quad = tries[t].quad;
+    ci = chunk_capacity(g, g->quad, tries[t].mb);
+    const size_t n_img = floats(g->img_stride * ci), n_sino = floats(g->sino_stride * ci);
+    const size_t n_imgT = g->quad ? floats((size_t)d.det_rows * d.det_cols * ci) : 0;
+    e = dmalloc((void **)&g->w_img, sizeof(float) * (n_img + n_imgT + 2 * n_sino));
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // not the next launch's error
+      continue;
+    }
+    g->w_imgT = g->quad ? g->w_img + n_img : nullptr;
+    g->w_sinoA = g->w_img + n_img + n_imgT;
+    g->w_sinoB = g->w_sinoA + n_sino;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "dc_setup_geometry: work area");
+  g->chunk_images = ci;
+  g->chunk_capacity = ci;
   if (g->quad) {
     const size_t H = d.det_rows, W = d.det_cols, ng = ci / 4;
     const L4Shape sh = l4_shape(d.det_rows, d.det_cols);
@@ -1342,7 +1359,8 @@ int alloc_workspace(dc_geometry *g) {
   }
   if (g->quad) {
     const size_t ng = ci / 4, n0 = 4 * (size_t)g->NSp, n1 = d.n_mu;
-    const int images = std::min(d.n_views, ci);
+    // of the usual work area: results do not depend on the memory that was free
+    const int images = std::min(d.n_views, chunk_capacity(g, true, QUAD_MB));
     g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, images);
     const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, images);
     g->q_nwx = b4.nwx;
