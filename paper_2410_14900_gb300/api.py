@@ -87,6 +87,7 @@ class Geometry:
         self._h = h
         self._lib = L
         self._px_per_mm = None
+        self.default_bp_nz = dc_geometry_get_tuning(self)["bp_nz"]
 
     def pixels_per_mm(self) -> float:
         """Detector pixels per mm at the volume's centre, in the middle view."""

@@ -25,10 +25,15 @@ def cache_path() -> str:
 
 
 def shape_key(geom: api.Geometry, dtype: str = "f32") -> str:
+    """What a plan depends on: the sizes, how large a voxel's footprint is, and
+    what the library planned itself (views with principal points of their own
+    take other filter kernels, with a smaller work area)."""
     d = geom.desc
-    # q4: timed with the four-image filter kernels, which want larger chunks
-    return "V{n_views}_H{det_rows}_W{det_cols}_mu{n_mu}_s{n_s}_vol{vol_z}x{vol_y}x{vol_x}".format(
-        **d) + f"_{dtype}_q4"
+    cap = api.dc_geometry_get_tuning(geom)["chunk_capacity"]
+    vox = "x".join(f"{v:.6g}" for v in d["voxel"])
+    return ("V{n_views}_H{det_rows}_W{det_cols}_mu{n_mu}_s{n_s}_vol{vol_z}x{vol_y}x{vol_x}".format(**d)
+            + f"_{dtype}_p{d['pitch']:.6g}_ds{d['ds']:.6g}_vox{vox}_px{geom.pixels_per_mm():.3g}"
+              f"_cap{cap}_nz{geom.default_bp_nz}")
 
 
 def _load():
@@ -66,13 +71,14 @@ def autotune(geom: api.Geometry, dtype: str = "f32", use_cache: bool = True,
     """Pick chunk_images and bp_nz for `geom`, apply them and return them
     (the backprojection timed with Kahan summation when `kahan`)."""
     key = shape_key(geom, dtype) + ("|kahan" if kahan else "")
+    cap = api.dc_geometry_get_tuning(geom)["chunk_capacity"]
     with _lock:
         db = _load() if use_cache else {}
     if key in db:
-        best = db[key]
+        best = dict(db[key])
+        best["chunk_images"] = min(best["chunk_images"], cap)
         api.dc_geometry_set_tuning(geom, best["chunk_images"], best["bp_nz"])
         return dict(best, cached=True)
-    cap = api.dc_geometry_get_tuning(geom)["chunk_capacity"]
     dev = torch.device("cuda", torch.cuda.current_device())
     g = torch.rand((1, geom.V, geom.H, geom.W), device=dev)
     gF = torch.empty(api.gF_shape(geom, 1, dtype), device=dev, dtype=api._DTYPES[dtype][1])
