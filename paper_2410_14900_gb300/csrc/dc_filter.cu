@@ -1282,7 +1282,7 @@ static int chunk_capacity(const dc_geometry *g, bool quad, long mb) {
 int quad_plan(dc_geometry *g) {
   const dc_geometry_desc &d = g->d;
   g->quad = 0;
-  if (getenv("DC_NO_QUAD") || d.det_rows < L4_RB || d.det_cols < L4_RB) return DC_OK;
+  if (d.det_rows < L4_RB || d.det_cols < L4_RB) return DC_OK;
   for (int i = 1; i < d.n_views; ++i)
     for (int c = 13; c <= 14; ++c)
       if (!(std::fabs(g->host_geo[(size_t)DC_VIEW_GEO_N * i + c] - g->host_geo[c]) < 1e-8))
