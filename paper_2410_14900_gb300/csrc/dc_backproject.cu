@@ -15,6 +15,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <string>
@@ -408,6 +409,12 @@ void bp_plan(dc_geometry *g) {
       ++all;
       if (front && vmax - vmin + 5.0 <= TB_BH) ++fit;
     }
+  }
+  {  // pixels per voxel at the volume's centre, in the middle view
+    const double *v = g->host_geo + (size_t)DC_VIEW_GEO_N * (d.n_views / 2);
+    double dep = 0.0;
+    for (int t = 0; t < 3; ++t) dep -= v[9 + t] * (d.vol_center[t] - v[t]);
+    g->bp_px = std::cbrt(dx * dy * dz) * v[12] / (dep * d.pitch);
   }
   const long boxes = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
                      ((d.vol_z + TB_NZ - 1) / TB_NZ);

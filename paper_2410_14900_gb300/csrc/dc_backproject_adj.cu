@@ -116,6 +116,14 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_bp3d_adj(BPAdjArgs a) {
 // Boxes are 32 deep, or 16 where 32-deep ones mostly do not fit the tile and
 // would scatter into global memory (214^2 x 178 voxels of 1.4 pixels, 86 views:
 // 5.2 ms, here 1.3).
+//
+// Three CTAs per SM take 80 registers and spill; two take 128 and do not.  For
+// voxels finer than 0.75 pixels, whose atomics meet in the same pixels, the
+// third CTA does not pay for that: 128^3 voxels, 200 views of 256 x 256, dense
+// gradient, three CTAs 1921, 1013 and 833 us at 0.1, 0.3 and 0.7 pixels per
+// voxel, two 1872, 952 and 783; behind a mask 1216, 784 and 749 against 1135,
+// 732 and 687.  At 1 pixel two cost 0.6 % behind a mask.
+constexpr double TA_FINE = 0.75;
 constexpr int TA_S = 68;  // row stride: 16-byte rows (69: 34.0 ms)
 static_assert(TA_S >= TB_BWW + 3, "a tile row holds the widest footprint from an aligned column");
 
@@ -130,8 +138,8 @@ __device__ __forceinline__ void red_add4(unsigned addr, int i00, int i01, int i1
       : "memory");
 }
 
-template <bool VEC4, int NZ>
-__global__ void __launch_bounds__(TB_TX *TB_TY, 3) k_bp3d_adj_tile(BPAdjArgs a, int split) {
+template <bool VEC4, int NZ, int CTAS>
+__global__ void __launch_bounds__(TB_TX *TB_TY, CTAS) k_bp3d_adj_tile(BPAdjArgs a, int split) {
   constexpr int NH = NZ / 2;  // a step takes voxels NH apart
   __shared__ __align__(16) int tiles[2][TB_BH * TA_S];
   __shared__ dc::BPView sv[TB_VCH];
@@ -481,8 +489,14 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
     while (split < 16 && 2 * split * boxes <= 456 && d.n_views >= 16 * split) split *= 2;
     // float4 atomics need 16-byte pixel quads
     const bool vec = (a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0;
-    auto kernel = nz == 32 ? (vec ? k_bp3d_adj_tile<true, 32> : k_bp3d_adj_tile<false, 32>)
-                           : (vec ? k_bp3d_adj_tile<true, 16> : k_bp3d_adj_tile<false, 16>);
+    const bool fine = g->bp_px < TA_FINE;
+    auto pick = [&](auto k32, auto k32f, auto k16, auto k16f) {
+      return nz == 32 ? (fine ? k32f : k32) : (fine ? k16f : k16);
+    };
+    auto kernel = vec ? pick(k_bp3d_adj_tile<true, 32, 3>, k_bp3d_adj_tile<true, 32, 2>,
+                             k_bp3d_adj_tile<true, 16, 3>, k_bp3d_adj_tile<true, 16, 2>)
+                      : pick(k_bp3d_adj_tile<false, 32, 3>, k_bp3d_adj_tile<false, 32, 2>,
+                             k_bp3d_adj_tile<false, 16, 3>, k_bp3d_adj_tile<false, 16, 2>);
     // whole items per launch, at most 65535 CTAs along z
     const int per = std::min(B, std::max(1, 65535 / (layers * split)));
     const size_t np = (size_t)d.n_views * d.det_rows * d.det_cols,

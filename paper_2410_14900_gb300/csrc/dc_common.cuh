@@ -152,6 +152,7 @@ struct dc_geometry {
   int l2_images;             // images whose per-image work area stays in L2
   int bp_nz;                 // voxels per thread along z in the backprojector (16, 32)
   int bp_fit32;              // footprints of 32-deep boxes (mostly) fit the staged tile
+  double bp_px;              // pixels per voxel
   int bp_split;              // CTAs (a cluster) that share the views of a 16-deep box
   size_t img_stride;         // floats per padded image  (H * Wp)
   size_t sino_stride;        // floats per padded sinogram (n_mu * NSp)
