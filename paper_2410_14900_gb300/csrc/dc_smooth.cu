@@ -24,7 +24,8 @@
 // sample once per period and every other sample twice) the filter A satisfies
 // A^T = D^-1 A D, exactly, also for lines shorter than the radius.
 //
-// Radii whose halo does not fit (above 320) take k_smooth_lines: `cw`
+// Radii whose halo does not fit (above 320), and few short lines (few_samples),
+// take k_smooth_lines: `cw`
 // neighbouring lines of one view whole in shared memory (cw = 16 columns for
 // the mu axis, whose elements are n_s apart; one contiguous row for the s
 // axis).  The forward pass gathers from a mirror-extended copy of the line;
@@ -328,6 +329,18 @@ int launch_lines(const SmoothLines &a, int views, cudaStream_t st) {
   return DC_OK;
 }
 
+// Few short lines leave the tiles' CTAs with nothing to overlap: what counts is
+// the time of one CTA, and that of k_smooth_lines, a few lines at a time, is
+// shorter.  16 views of 90 x 64, radius 3: 11.1 us with it, 14.4 with tiles
+// (radius 60: 23.1 and 22.6); 48 views 16.3 and 14.5; one view of 360 x 256 20.1
+// and 17.1, six of 250 x 80 with radius 15 21.3 and 19.6.  Its transpose folds the halo back and so takes small radii only
+// (4 views of 90 x 64: radius 15 13.4 and 17.6, radius 60 32.5 and 25.2).
+bool few_samples(int V, int n_mu, int n_s, int radius, int adjoint) {
+  const double n = (double)V * n_mu * n_s;
+  return V <= 65535 && n <= 1 << 17 && std::max(n_mu, n_s) <= 224 &&
+         (adjoint ? radius <= 16 : n * (2 * radius + 1) <= 1 << 23);
+}
+
 // lines per CTA along mu: the widest power of two (<= 16) whose staging fits
 int mu_log_width(int n_mu, int R, int adjoint) {
   for (int l = 4; l >= 0; --l)
@@ -375,7 +388,7 @@ extern "C" int dc_gauss_smooth(int V, int n_mu, int n_s, float sigma, int radius
   s_axis.in = in;
   s_axis.out = work;
   int rc;
-  if (radius <= ST_MAX_R) {
+  if (radius <= ST_MAX_R && !few_samples(V, n_mu, n_s, radius, ad)) {
     if ((rc = launch_tile(s_axis, V, nullptr, st))) return rc;
     mu_axis.in = work;
     mu_axis.out = out;
