@@ -51,7 +51,7 @@ __device__ __forceinline__ float powi(float x, int m) {
   return r;
 }
 
-// A CTA takes CR_MU angles of one view; the orbit relative to a_i lives in
+// A CTA takes up to CR_MU angles of one view; the orbit relative to a_i lives in
 // shared memory, once for all of them.  A warp takes 32 neighbouring s-bins of
 // one angle (lane = plane).
 //
@@ -63,9 +63,9 @@ __device__ __forceinline__ float powi(float x, int m) {
 // pairs whose two views are not both positive or both negative are looked at
 // plane by plane, in the same order and with the same arithmetic (1.66 ms).
 // A view within the rounding of f of zero at an end counts as neither.
-constexpr int CR_MU = 16;
+constexpr int CR_MU = 16;  // at most: fewer where the grid would not fill the GPU
 
-__global__ void __launch_bounds__(CR_THREADS) k_crofton(CroftonArgs a) {
+__global__ void __launch_bounds__(CR_THREADS) k_crofton(CroftonArgs a, int n_ang) {
   extern __shared__ float4 orb[];  // [V] (a_j - a_i, c_j), then [V] (v_j, 0)
   const int i = blockIdx.y;
   const double *gi = a.geo + (size_t)DC_VIEW_GEO_N * i;
@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(CR_THREADS) k_crofton(CroftonArgs a) {
   }
   const float4 vi = vt[i];
   const float ci = orb[i].w;
-  const int nch = (a.n_s + 31) >> 5, m0 = blockIdx.x * CR_MU;
-  const int items = min(CR_MU, a.n_mu - m0) * nch;
+  const int nch = (a.n_s + 31) >> 5, m0 = blockIdx.x * n_ang;
+  const int items = min(n_ang, a.n_mu - m0) * nch;
   for (int w = threadIdx.x >> 5; w < items; w += CR_THREADS / 32) {
     const int m = m0 + w / nch, k0 = (w % nch) * 32, k = k0 + lane;
     const dc::MuRec mr = a.mu[m];
@@ -194,8 +194,13 @@ extern "C" int dc_crofton_weights(const dc_geometry *g, int n_seg, const int *se
   DC_CUDA(cudaFuncSetAttribute(k_crofton, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                200 * 1024));
   // the grid's y limit is 65535; shared memory allows 6400 views
-  dim3 grid((d.n_mu + CR_MU - 1) / CR_MU, d.n_views);
-  k_crofton<<<grid, CR_THREADS, smem, st>>>(a);
+  // few views: fewer angles per CTA until two CTAs per SM have some (16 views,
+  // 90 x 64 planes: 8.6 us with 16 angles, 6.5 with 2; 6 views, 720 x 512: 43 and
+  // 34)
+  int n_ang = CR_MU;
+  while (n_ang > 1 && (long)((d.n_mu + n_ang - 1) / n_ang) * d.n_views < 304) n_ang /= 2;
+  dim3 grid((d.n_mu + n_ang - 1) / n_ang, d.n_views);
+  k_crofton<<<grid, CR_THREADS, smem, st>>>(a, n_ang);
   DC_CHECK_LAUNCH("k_crofton");
   return DC_OK;
 }
