@@ -1,6 +1,8 @@
 """The storage form of a g^F that only the next backprojection reads: which
 calls take FP32 pairs, that both forms agree, and what happens where the pairs,
 twice the memory, do not fit."""
+import gc
+
 import pytest
 import torch
 
@@ -49,18 +51,22 @@ def test_pairs_that_do_not_fit_give_way():
     gF, _ = api.dc_filter(geom, g, None, "f32")
     ref = api.dc_backproject(geom, gF)
     del gF
+    gc.collect()
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
-    # room for g^F in FP32 (42 MB) and the volume (16 MB), not for the pairs (84 MB)
+    # room for g^F in FP32 (42 MB) and the volume (16 MB), not for the pairs (84
+    # MB); a pool of their own, where no block of earlier tests is free
     room = torch.cuda.memory_reserved() + (72 << 20)
     total = torch.cuda.get_device_properties(0).total_memory
     torch.cuda.set_per_process_memory_fraction(room / total)
     try:
-        vol = api.reconstruct(geom, g)
+        with torch.cuda.use_mem_pool(torch.cuda.MemPool()):
+            vol = api.reconstruct(geom, g)
         same = torch.equal(vol, ref)
         del vol
         torch.cuda.empty_cache()
-        net = reconstruct(g, None, geom)
+        with torch.cuda.use_mem_pool(torch.cuda.MemPool()):
+            net = reconstruct(g, None, geom)
         assert same and torch.equal(net, ref)
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
