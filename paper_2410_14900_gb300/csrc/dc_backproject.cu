@@ -422,14 +422,14 @@ void bp_plan(dc_geometry *g) {
   const long boxes = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
                      ((d.vol_z + TB_NZ - 1) / TB_NZ);
   g->bp_fit32 = fit >= all * 0.95;
-  g->bp_nz = (!g->bp_fit32 || boxes < 152) ? 16 : 32;
+  g->bp_nz = (!g->bp_fit32 || boxes < g->sms) ? 16 : 32;
   // views split over clusters where 16-deep boxes are fewer than the SMs: as
   // many CTAs as two per SM hold, at least 8 views each (64 boxes, 64 views:
   // 57 us unsplit, 33 us split by four)
   const long boxes16 = (long)((d.vol_x + TB_TX - 1) / TB_TX) * ((d.vol_y + TB_TY - 1) / TB_TY) *
                        ((d.vol_z + 15) / 16);
   g->bp_split = 1;
-  while (g->bp_split < 8 && 2 * g->bp_split * boxes16 <= 304 && d.n_views >= 16 * g->bp_split)
+  while (g->bp_split < 8 && g->bp_split * boxes16 <= g->sms && d.n_views >= 16 * g->bp_split)
     g->bp_split *= 2;
 }
 

@@ -486,7 +486,7 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
     // views each
     const long boxes = (long)gridt.x * gridt.y * layers * B;
     int split = 1;
-    while (split < 16 && 2 * split * boxes <= 456 && d.n_views >= 16 * split) split *= 2;
+    while (split < 16 && 2 * split * boxes <= 3 * g->sms && d.n_views >= 16 * split) split *= 2;
     // float4 atomics need 16-byte pixel quads
     const bool vec = (a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0;
     const bool fine = g->bp_px < TA_FINE;

@@ -146,6 +146,7 @@ struct dc_geometry {
   int n_groups;
   int n_groups_branch0;
   int mg;                    // max angles per group
+  int sms;                   // SMs of the device, for the plans
   // work area
   int chunk_images;          // images (view x batch item) per chunk
   int chunk_capacity;        // images the work area was sized for

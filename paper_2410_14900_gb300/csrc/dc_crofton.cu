@@ -198,7 +198,7 @@ extern "C" int dc_crofton_weights(const dc_geometry *g, int n_seg, const int *se
   // 90 x 64 planes: 8.6 us with 16 angles, 6.5 with 2; 6 views, 720 x 512: 43 and
   // 34)
   int n_ang = CR_MU;
-  while (n_ang > 1 && (long)((d.n_mu + n_ang - 1) / n_ang) * d.n_views < 304) n_ang /= 2;
+  while (n_ang > 1 && (long)((d.n_mu + n_ang - 1) / n_ang) * d.n_views < 2 * g->sms) n_ang /= 2;
   dim3 grid((d.n_mu + n_ang - 1) / n_ang, d.n_views);
   k_crofton<<<grid, CR_THREADS, smem, st>>>(a, n_ang);
   DC_CHECK_LAUNCH("k_crofton");

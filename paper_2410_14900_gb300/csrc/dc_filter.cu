@@ -1302,7 +1302,7 @@ int quad_plan(dc_geometry *g) {
       if (ng) most = std::max(most, (nb[br] + ng - 1) / ng);
     }
     const int rounds = (most * nch + L4_WARPS - 1) / L4_WARPS;
-    const double cost = ((groups * quads + 151) / 152) * (rounds + over);
+    const double cost = ((groups * quads + g->sms - 1) / g->sms) * (rounds + over);
     if (!g->quad || cost < best) {
       best = cost;
       g->q_mg = mg;
@@ -1361,8 +1361,8 @@ int alloc_workspace(dc_geometry *g) {
     const size_t ng = ci / 4, n0 = 4 * (size_t)g->NSp, n1 = d.n_mu;
     // of the usual work area: results do not depend on the memory that was free
     const int images = std::min(d.n_views, chunk_capacity(g, true, QUAD_MB));
-    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, images);
-    const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, images);
+    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, images, g->sms);
+    const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, images, g->sms);
     g->q_nwx = b4.nwx;
     const int lwb = b4.lwb;
     if (!encode_map_f32(&g->q_tm_sinoA, g->w_sinoA, n0, n1, ng, 4 * lwb, 1) ||

@@ -587,7 +587,7 @@ inline long b4_tiles(int H, int W, const B4Shape &s, int RY, int images) {
 // CTA per SM, 775 in 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds
 // of 256 x 8, 655 in 5 of 128 x 16.  With 2 rows (grids of less than a wave) it
 // is the pixels computed, those outside the detector too.
-inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int images) {
+inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int images, int sms) {
   const double alone = b4_taps(pitch, ds) == 2 ? 1.28 : 1.13;
   B4Shape best = {};
   double least = -1.0;
@@ -596,7 +596,7 @@ inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int image
     const B4Shape s = b4_arrange(order[i], pitch, ds, RY);
     const size_t sm = b4_smem(s);
     if (i > 0 && sm > (size_t)B4_SMEM_MAX) continue;
-    const long tiles = b4_tiles(H, W, s, RY, images), n = (tiles + 151) / 152;
+    const long tiles = b4_tiles(H, W, s, RY, images), n = (tiles + sms - 1) / sms;
     const double cost = RY == 2 ? (double)tiles
                         : sm <= (size_t)B4_SMEM_TWO ? 2.0 * (n / 2) + alone * (n % 2)
                                                     : alone * n;
@@ -613,8 +613,8 @@ inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int image
 // 90 views of 128 x 128, 184 tiles: 168 against 158).  A property of the
 // geometry, so that an image's result does not depend on the chunk or batch
 // that it comes in.
-inline int b4_rows(int H, int W, double pitch, double ds, int images) {
-  return b4_tiles(H, W, b4_shape(H, W, pitch, ds, 8, images), 8, images) < 152 ? 2 : 8;
+inline int b4_rows(int H, int W, double pitch, double ds, int images, int sms) {
+  return b4_tiles(H, W, b4_shape(H, W, pitch, ds, 8, images, sms), 8, images) < sms ? 2 : 8;
 }
 
 // 8 rows per thread want the registers of two CTAs per SM (496 images of 384 x

@@ -297,6 +297,7 @@ int dc_setup_geometry(const dc_geometry_desc *desc, const double *P, const doubl
     cudaError_t e_ = (call);                                     \
     if (e_ != cudaSuccess) return cleanup(dc::cuda_fail(e_, #call)); \
   } while (0)
+  SETUP_CUDA(cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
   SETUP_CUDA(dc::dmalloc((void **)&g->geo64, sizeof(double) * GN * V));
   SETUP_CUDA(dc::dmalloc((void **)&g->bpv, sizeof(dc::BPView) * V));
   SETUP_CUDA(dc::dmalloc((void **)&g->fv, sizeof(dc::FView) * V));
