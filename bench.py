@@ -441,7 +441,8 @@ def train_step_512_measure(args, dev, L):
                               device=dev, dtype=torch.float32)[None].contiguous()
     tgt = synth.phantom_volume(blobs, w.vol_shape, w.voxel, device=dev)[None]
     t = api.dc_geometry_get_tuning(geom)
-    per_img = 4 * (w.det_rows * ((w.det_cols + 3) // 4 * 4)
+    # the image, its transpose and two sinograms
+    per_img = 4 * (w.det_rows * ((w.det_cols + 3) // 4 * 4) + w.det_rows * w.det_cols
                    + 2 * w.n_mu * ((w.n_s + 3) // 4 * 4))
     work_bytes = int(t["chunk_capacity"]) * per_img
     stream = torch.cuda.current_stream()

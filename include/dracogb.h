@@ -62,7 +62,9 @@ extern "C" {
 
 /* storage types of the filtered projections g^F */
 #define DC_F32 0
-#define DC_BF16 1             /* round-to-nearest-even                      */
+#define DC_BF16 1             /* round-to-nearest-even; filtered one image at
+                                 a time (the others four at once), the bits
+                                 of earlier versions                        */
 #define DC_F16 2              /* with a per-view power-of-two scale         */
 /* FP32 (value, right difference) pairs: pixel (r, c) of g^F is stored as
  * the two floats g[r][c] and g[r][c+1] - g[r][c] (g[r][W] = 0), i.e.

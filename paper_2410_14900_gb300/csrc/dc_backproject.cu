@@ -1,6 +1,6 @@
 // dc_backproject.cu -- voxel-driven cone-beam backprojection A3d^T of the
 // filtered projections (Ye et al., DRACO, Eq. 5 and the last layer of
-// Eq. 12), optional ReLU (Sec. 2.3), and its transpose.
+// Eq. 12), optional ReLU (Sec. 2.3), and the batched reconstruction.
 //
 //   f(X) = sum_i bilinear(g^F_i, P_i X) / |X - a_i|^2
 //

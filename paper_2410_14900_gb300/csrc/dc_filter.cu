@@ -1083,18 +1083,20 @@ Chunking chunking(const dc_geometry *g, int B, int view_limit = 0) {
   return c;
 }
 
-// Four images at once cost about the time of two single ones (their step
-// runs at more than twice the rate), so single-image chunks keep the
-// per-image kernel.  The rule looks at the plan of the whole call, not at a
-// chunk, so that every image of a call takes the same path.
+// Chunks planned for one image (view_chunk or chunk_images of 1) keep the
+// per-image kernels.  The rule looks at the plan of the whole call, not at a
+// chunk, so that every image of a call takes the same path; a group that is not
+// full costs what a full one does, which is still less than one image alone
+// (filter of one image: 64 x 64, 180 angles 160 us per image, 57 as a group;
+// 384 x 512, 720 angles 689 and 419).
 bool use_quad(const dc_geometry *g, int bc, int cv) { return g->quad && bc * cv >= 2; }
 
-// BF16 storage keeps the per-image kernels.  The two paths' FP32 results
+// BF16 storage keeps the per-image kernels, so that a stored g^F and what is
+// reconstructed from it stay the bits they were.  The two paths' FP32 results
 // differ by their rounding (5e-6 relative), which turns 0.1 % of the BF16
-// roundings the other way, each by 2^-8 of its value; the reconstructions that
-// differ by that (2.2e-5 relative, 1.5e-3 at most) are further apart than FP32
-// results of one input may be from release to release (2e-5, 8e-4).  FP16's
-// roundings, eight times finer, stay inside (5e-6, 6e-5).
+// roundings the other way, each by 2^-8 of its value: reconstructions 2.2e-5
+// apart (relative L2; 1.5e-3 at most), equally far from FP64.  FP16's roundings
+// are eight times finer (5e-6, 6e-5).
 bool quad_storage(int dtype) { return dtype != DC_BF16; }
 
 // ------------------------------------------------ batched persistent filter

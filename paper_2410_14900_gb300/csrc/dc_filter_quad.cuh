@@ -25,7 +25,8 @@
 // 512 lines: 37.1 ms with the per-image kernel (7.0 steps per clock and SM);
 // here 22.3 ms with 16 warps and a CTA barrier per band (data pipe 65 %, waits
 // for shared memory: too few warps), 20.7 ms with this split, 21.2 with 24
-// warps (80 registers), 21.6 with 16 (128).  12.1 steps per clock and SM.
+// warps (80 registers), 21.6 with 16 (128), all before the groups were planned
+// by waves; now 20.3 ms, 12.8 steps per clock and SM.
 constexpr int L4_WARPS = 19;
 constexpr int L4_THREADS = 32 * L4_WARPS + 32;
 constexpr int L4_T = 6;                  // tasks (angle, 32 lines) per warp
@@ -442,7 +443,7 @@ __global__ void __launch_bounds__(L4_THREADS, 1)
 }
 
 // the last step of the filter's reverse mode from a kept S (k_adj_from_s) on
-// quad sinograms: a CTA takes AS_ROWS angles of four images
+// quad sinograms: a CTA takes AS4_ROWS angles of four images
 constexpr int AS4_ROWS = 2;
 __global__ void __launch_bounds__(256) k_adj_from_s4(LineArgs a, const float *__restrict__ S) {
   extern __shared__ __align__(16) float4 ys4[];  // [AS4_ROWS][NSp]
