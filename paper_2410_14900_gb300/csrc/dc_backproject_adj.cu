@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_bp3d_adj(BPAdjArgs a) {
 // third CTA does not pay for that: 128^3 voxels, 200 views of 256 x 256, dense
 // gradient, three CTAs 1921, 1013 and 833 us at 0.1, 0.3 and 0.7 pixels per
 // voxel, two 1872, 952 and 783; behind a mask 1216, 784 and 749 against 1135,
-// 732 and 687.  At 1 pixel two cost 0.6 % behind a mask.
+// 732 and 687.  At 1 pixel two cost 0.6 % behind a mask; where three hold every box
+// at once (100 x 100 x 33 voxels, 0.5 pixels: 322 us) two cost 25 %.
 constexpr double TA_FINE = 0.75;
 constexpr int TA_S = 68;  // row stride: 16-byte rows (69: 34.0 ms)
 static_assert(TA_S >= TB_BWW + 3, "a tile row holds the widest footprint from an aligned column");
@@ -489,7 +490,7 @@ extern "C" int dc_backproject_adjoint(const dc_geometry *g, int B, const float *
     while (split < 16 && 2 * split * boxes <= 3 * g->sms && d.n_views >= 16 * split) split *= 2;
     // float4 atomics need 16-byte pixel quads
     const bool vec = (a.W & 3) == 0 && ((uintptr_t)grad_gF & 15) == 0;
-    const bool fine = g->bp_px < TA_FINE;
+    const bool fine = g->bp_px < TA_FINE && split * boxes > 3 * g->sms;
     auto pick = [&](auto k32, auto k32f, auto k16, auto k16f) {
       return nz == 32 ? (fine ? k32f : k32) : (fine ? k16f : k16);
     };

@@ -14,10 +14,11 @@ pytestmark = pytest.mark.gpu
 
 
 # on both sides of the line (pitch 1.5, 1.6 times the voxel); rows of whole
-# quads and not; volumes within a box, one voxel beyond it and of whole boxes
+# quads and not; volumes within a box, one voxel beyond it, of whole boxes and
+# of more boxes than three CTAs per SM hold at once (the two-CTA kernel)
 @pytest.mark.parametrize("voxel", [0.05, 0.3, 0.70, 0.71])
 @pytest.mark.parametrize("W", [40, 41])
-@pytest.mark.parametrize("n,nz", [(9, 5), (33, 33), (32, 64)])
+@pytest.mark.parametrize("n,nz", [(9, 5), (33, 33), (32, 64), (145, 65)])
 @pytest.mark.parametrize("relu", [False, True])
 def test_fine_voxels(voxel, W, n, nz, relu):
     V, H, p = 34, 30, 1.5
