@@ -65,7 +65,9 @@ __device__ __forceinline__ int mirror_of(int p, int n) {
   return p < n ? p : T - p;
 }
 
-__global__ void __launch_bounds__(SM_THREADS) k_smooth_lines(SmoothLines a) {
+// `through` (mu axis): the array whose entry `lines` of every row passes into a.out
+__global__ void __launch_bounds__(SM_THREADS)
+    k_smooth_lines(SmoothLines a, const float *__restrict__ through) {
   extern __shared__ float sm[];
   const int R = a.R, n = a.n, cw = 1 << a.lcw, cm = cw - 1;
   const int ntap = 2 * R + 1;
@@ -76,6 +78,11 @@ __global__ void __launch_bounds__(SM_THREADS) k_smooth_lines(SmoothLines a) {
   float *dst = a.out + (size_t)v * a.vstride + (size_t)l0 * a.ls;
   const int tid = threadIdx.x;
 
+  if (through && blockIdx.x == 0)
+    for (int j = tid; j < n; j += SM_THREADS) {
+      const size_t o = (size_t)v * a.vstride + (size_t)j * a.es + (size_t)a.lines * a.ls;
+      a.out[o] = through[o];
+    }
   for (int t = tid; t < ntap; t += SM_THREADS) {
     const float d = (float)(t - R);
     w[t] = expf(-0.5f * d * d / (a.sigma * a.sigma));
@@ -313,7 +320,7 @@ size_t smem_floats(int n, int R, int lcw, int adjoint) {
          ((size_t)1 << lcw) * (size_t)(adjoint ? (2 * n + 6 * R) : (n + 2 * R));
 }
 
-int launch_lines(const SmoothLines &a, int views, cudaStream_t st) {
+int launch_lines(const SmoothLines &a, int views, const float *through, cudaStream_t st) {
   const int cw = 1 << a.lcw;
   const size_t smem = smem_floats(a.n, a.R, a.lcw, a.adjoint) * sizeof(float);
   static bool attr_done = false;
@@ -324,7 +331,7 @@ int launch_lines(const SmoothLines &a, int views, cudaStream_t st) {
   }
   dim3 grid((unsigned)((a.lines + cw - 1) / cw), (unsigned)views);
   dc::ProfScope ps(dc::KID_SMOOTH, st);
-  k_smooth_lines<<<grid, SM_THREADS, smem, st>>>(a);
+  k_smooth_lines<<<grid, SM_THREADS, smem, st>>>(a, through);
   DC_CHECK_LAUNCH("k_smooth_lines");
   return DC_OK;
 }
@@ -394,13 +401,8 @@ extern "C" int dc_gauss_smooth(int V, int n_mu, int n_s, float sigma, int radius
     mu_axis.out = out;
     return launch_tile(mu_axis, V, in, st);
   }
-  rc = launch_lines(s_axis, V, st);
-  if (rc != DC_OK) return rc;
+  if ((rc = launch_lines(s_axis, V, nullptr, st))) return rc;
   mu_axis.in = work;
   mu_axis.out = out;
-  rc = launch_lines(mu_axis, V, st);
-  if (rc != DC_OK) return rc;
-  DC_CUDA(cudaMemcpy2DAsync(out + ns1, sizeof(float) * n_s, in + ns1, sizeof(float) * n_s,
-                            sizeof(float), (size_t)V * n_mu, cudaMemcpyDeviceToDevice, st));
-  return DC_OK;
+  return launch_lines(mu_axis, V, in, st);
 }
