@@ -339,7 +339,7 @@ int launch_lines(const SmoothLines &a, int views, const float *through, cudaStre
 // Few short lines leave the tiles' CTAs with nothing to overlap: what counts is
 // the time of one CTA, and that of k_smooth_lines, a few lines at a time, is
 // shorter.  16 views of 90 x 64, radius 3: 11.1 us with it, 14.4 with tiles
-// (radius 60: 23.1 and 22.6); 48 views 16.3 and 14.5; one view of 360 x 256 20.1
+// (radius 60: 23.1 and 22.6; about 1 us less since no copy follows it); 48 views 16.3 and 14.5; one view of 360 x 256 20.1
 // and 17.1, six of 250 x 80 with radius 15 21.3 and 19.6.  Its transpose folds the halo back and so takes small radii only
 // (4 views of 90 x 64: radius 15 13.4 and 17.6, radius 60 32.5 and 25.2).
 bool few_samples(int V, int n_mu, int n_s, int radius, int adjoint) {
