@@ -1362,9 +1362,10 @@ int alloc_workspace(dc_geometry *g) {
   if (g->quad) {
     const size_t ng = ci / 4, n0 = 4 * (size_t)g->NSp, n1 = d.n_mu;
     // of the usual work area: results do not depend on the memory that was free
-    const int images = std::min(d.n_views, chunk_capacity(g, true, QUAD_MB));
-    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, images, g->sms);
-    const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, images, g->sms);
+    const int chunk = chunk_capacity(g, true, QUAD_MB);
+    g->q_ry = b4_rows(d.det_rows, d.det_cols, d.pitch, d.ds, d.n_views, chunk, g->sms);
+    const B4Shape b4 = b4_shape(d.det_rows, d.det_cols, d.pitch, d.ds, g->q_ry, d.n_views, chunk,
+                                g->sms);
     g->q_nwx = b4.nwx;
     const int lwb = b4.lwb;
     if (!encode_map_f32(&g->q_tm_sinoA, g->w_sinoA, n0, n1, ng, 4 * lwb, 1) ||

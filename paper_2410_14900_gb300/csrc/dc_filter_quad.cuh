@@ -578,29 +578,42 @@ inline long b4_tiles(int H, int W, const B4Shape &s, int RY, int images) {
   return (long)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * ((images + 3) / 4);
 }
 
-// The warps' arrangement with the least time for `images` images among those
-// whose stages an SM holds (the squarest of equals: the smallest window).  At
-// ds >= pitch / 3 the squarest one always fits (112 KB); 256 x 8 tiles want 140
-// KB at ds = pitch, 288 at pitch / 2.  With 8 rows per thread that time is what
-// an SM's share of the tiles takes: two CTAs together 2 units, one alone, or at
-// a time because two do not fit, 1.28 (two taps) or 1.13 (more): 96 images,
-// 180 angles, ds = pitch: 360 x 512 974 us in 15 rounds of 256 x 8 tiles, one
-// CTA per SM, 775 in 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds
-// of 256 x 8, 655 in 5 of 128 x 16.  With 2 rows (grids of less than a wave) it
-// is the pixels computed, those outside the detector too.
-inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int images, int sms) {
-  const double alone = b4_taps(pitch, ds) == 2 ? 1.28 : 1.13;
+// What an SM's share of the tiles of `items` batch items of all views takes, in
+// chunks of `chunk` images: two CTAs together 2 units, one alone, or at a time
+// because two do not fit, 1.28 (two taps) or 1.13 (more).
+inline double b4_rounds(int H, int W, const B4Shape &s, int taps, int views, int items, int chunk,
+                        int sms) {
+  const double alone = taps == 2 ? 1.28 : 1.13;
+  const int bc = std::min(items, chunk), cv = std::min(views, std::max(1, chunk / bc));
+  auto time = [&](int v) {
+    const long n = (b4_tiles(H, W, s, 8, v * bc) + sms - 1) / sms;
+    return b4_smem(s) <= (size_t)B4_SMEM_TWO ? 2.0 * (n / 2) + alone * (n % 2) : alone * n;
+  };
+  return (views / cv) * time(cv) + (views % cv ? time(views % cv) : 0.0);
+}
+
+// The warps' arrangement with the least time among those whose stages an SM
+// holds (the squarest of equals: the smallest window).  At ds >= pitch / 3 the
+// squarest one always fits (112 KB); 256 x 8 tiles want 140 KB at ds = pitch, 288
+// at pitch / 2.  With 8 rows per thread that time is b4_rounds per item, over
+// batches of one to four items, fewer items counting more: 96 images, 180 angles,
+// ds = pitch: 360 x 512 974 us in 15 rounds of 256 x 8 tiles, one CTA per SM, 775
+// in 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds of 256 x 8, 655 in
+// 5 of 128 x 16.  (Judged by one item alone, 30 views of 300 x 400 take 4 % longer
+// with three.)  With 2 rows (grids of less than a wave) it is the pixels
+// computed, those outside the detector too.
+inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int views, int chunk,
+                        int sms) {
   B4Shape best = {};
   double least = -1.0;
-  const int order[4] = {2, 1, 4, 8};
+  const int order[4] = {2, 1, 4, 8}, taps = b4_taps(pitch, ds);
   for (int i = 0; i < 4; ++i) {
     const B4Shape s = b4_arrange(order[i], pitch, ds, RY);
-    const size_t sm = b4_smem(s);
-    if (i > 0 && sm > (size_t)B4_SMEM_MAX) continue;
-    const long tiles = b4_tiles(H, W, s, RY, images), n = (tiles + sms - 1) / sms;
-    const double cost = RY == 2 ? (double)tiles
-                        : sm <= (size_t)B4_SMEM_TWO ? 2.0 * (n / 2) + alone * (n % 2)
-                                                    : alone * n;
+    if (i > 0 && b4_smem(s) > (size_t)B4_SMEM_MAX) continue;
+    double cost = 0.0;
+    if (RY == 2) cost = (double)b4_tiles(H, W, s, RY, 4);
+    else
+      for (int b = 1; b <= 4; ++b) cost += b4_rounds(H, W, s, taps, views, b, chunk, sms) / (b * b);
     if (least < 0.0 || cost < least) {
       least = cost;
       best = s;
@@ -614,8 +627,9 @@ inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int image
 // 90 views of 128 x 128, 184 tiles: 168 against 158).  A property of the
 // geometry, so that an image's result does not depend on the chunk or batch
 // that it comes in.
-inline int b4_rows(int H, int W, double pitch, double ds, int images, int sms) {
-  return b4_tiles(H, W, b4_shape(H, W, pitch, ds, 8, images, sms), 8, images) < sms ? 2 : 8;
+inline int b4_rows(int H, int W, double pitch, double ds, int views, int chunk, int sms) {
+  const B4Shape s = b4_shape(H, W, pitch, ds, 8, views, chunk, sms);
+  return b4_tiles(H, W, s, 8, std::min(views, chunk)) < sms ? 2 : 8;
 }
 
 // 8 rows per thread want the registers of two CTAs per SM (496 images of 384 x
