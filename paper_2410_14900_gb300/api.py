@@ -10,6 +10,7 @@ runs in the CUDA library.  Layouts (Ye et al., DRACO, Eq. 12):
 from __future__ import annotations
 
 import ctypes
+import math
 from typing import Optional
 
 import numpy as np
@@ -95,7 +96,8 @@ class Geometry:
             v = dc_get_view_geometry(self)[self.V // 2].tolist()
             c = self.desc.get("vol_center", (0.0, 0.0, 0.0))
             depth = sum((v[t] - c[t]) * v[9 + t] for t in range(3))
-            self._px_per_mm = v[12] / (depth * self.desc["pitch"])
+            # (a centre in the source's own plane is magnified without bound)
+            self._px_per_mm = v[12] / (depth * self.desc["pitch"]) if depth > 0 else math.inf
         return self._px_per_mm
 
     @property

@@ -43,6 +43,18 @@ def test_form_and_agreement(V, H, W, n, voxel, form):
     assert rel_l2(vol.double().cpu().numpy(), ref.double().cpu().numpy()) < 1e-5
 
 
+def test_a_centre_beside_the_source():
+    """The middle view's source level with the volume's centre: no scale."""
+    o = synth.circle_orbit(64)
+    desc = dict(n_views=64, det_rows=256, det_cols=256, n_mu=8, n_s=64, pitch=1.0, ds=4.0, vol_x=32,
+                vol_y=32, vol_z=32, voxel=(1.0,) * 3, closed_orbit=1)
+    a = o.sources[32]
+    desc["vol_center"] = (float(a[0]), float(a[1]), float(a[2]))
+    geom = api.Geometry(desc, synth.projection_matrices(o, 256, 256, 1.0), o.vdl)
+    assert geom.pixels_per_mm() > 1e6
+    assert api.transient_dtype(geom, 1) == "f32"
+
+
 def test_pairs_that_do_not_fit_give_way():
     V, H, W, n = 160, 256, 256, 160
     geom = _geometry(V, H, W, n, 0.9)
