@@ -593,23 +593,36 @@ inline double b4_rounds(int H, int W, const B4Shape &s, int taps, int views, int
 }
 
 // The warps' arrangement with the least time among those whose stages an SM
-// holds (the squarest of equals: the smallest window).  At ds >= pitch / 3 the
-// squarest one always fits (112 KB); 256 x 8 tiles want 140 KB at ds = pitch, 288
-// at pitch / 2.  With 8 rows per thread that time is b4_rounds per item, over
-// batches of one to four items, fewer items counting more: 96 images, 180 angles,
-// ds = pitch: 360 x 512 974 us in 15 rounds of 256 x 8 tiles, one CTA per SM, 775
-// in 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds of 256 x 8, 655 in
-// 5 of 128 x 16.  (Judged by one item alone, 30 views of 300 x 400 take 4 % longer
-// with three.)  With 2 rows (grids of less than a wave) it is the pixels
-// computed, those outside the detector too.
+// holds (the squarest of equals: the smallest window) and no wider than the one
+// with the fewest pixels outside the detector: a position is rounded at its
+// distance from the tile's first column, so width costs accuracy (filter of 256
+// images of 58 x 80: 1.5e-6 relative L2 from FP64 with 64 x 32 tiles, 1.1e-6 with
+// 32 x 64), which is paid for fewer pixels only.  At ds >= pitch / 3 the two
+// narrow ones always fit (112 KB); 256 x 8 tiles want 140 KB at ds = pitch, 288 at
+// pitch / 2.  With 8 rows per thread the time is b4_rounds per item, over batches
+// of one to four items, fewer items counting more: 96 images, 180 angles, ds =
+// pitch: 360 x 512 974 us in 15 rounds of 256 x 8 tiles, one CTA per SM, 775 in
+// 128 x 16 tiles; at 0.8 pitch 200 x 256 590 us in 4 rounds of 256 x 8, 655 in 5 of
+// 128 x 16.  (Judged by one item alone, 30 views of 300 x 400 take 4 % longer with
+// three.)  With 2 rows (grids of less than a wave) it is the pixels computed,
+// those outside the detector too.
 inline B4Shape b4_shape(int H, int W, double pitch, double ds, int RY, int views, int chunk,
                         int sms) {
+  const int order[4] = {2, 1, 4, 8}, taps = b4_taps(pitch, ds);
+  long fewest = -1;
+  int widest = 0;
+  for (int nwx : order) {
+    const long tiles = b4_tiles(H, W, b4_arrange(nwx, pitch, ds, RY), RY, 4);
+    if (fewest < 0 || tiles < fewest) {
+      fewest = tiles;
+      widest = nwx;
+    }
+  }
   B4Shape best = {};
   double least = -1.0;
-  const int order[4] = {2, 1, 4, 8}, taps = b4_taps(pitch, ds);
-  for (int i = 0; i < 4; ++i) {
-    const B4Shape s = b4_arrange(order[i], pitch, ds, RY);
-    if (i > 0 && b4_smem(s) > (size_t)B4_SMEM_MAX) continue;
+  for (int nwx : order) {
+    const B4Shape s = b4_arrange(nwx, pitch, ds, RY);
+    if (nwx > widest || (nwx > 2 && b4_smem(s) > (size_t)B4_SMEM_MAX)) continue;
     double cost = 0.0;
     if (RY == 2) cost = (double)b4_tiles(H, W, s, RY, 4);
     else
