@@ -38,3 +38,18 @@ def test_more_views_than_a_grid_holds():
     W = torch.rand((V, 1, 2), device="cuda")
     # one sample a line, whose three taps sum to 1 but for their rounding
     assert torch.allclose(api.dc_gauss_smooth(W, 2.0, 1), W, rtol=1e-6, atol=0.0)
+
+
+# A running sum of the taps rounds 2 radius times, one way for neighbouring sums,
+# and scales every output by its error (4e-7 for the two axes at radius 60).  In 32
+# parts it rounds some ten times: with the taps' own rounding (2 units of 6e-8)
+# and the FMAs', which average out, 5 units are not reached.
+@pytest.mark.parametrize("views", [4, 30])
+@pytest.mark.parametrize("adjoint", [False, True])
+@pytest.mark.parametrize("sigma,radius", [(5.0, 15), (20.0, 60)])
+def test_taps_sum_to_one(views, adjoint, sigma, radius):
+    rng = np.random.default_rng(radius)
+    W = rng.uniform(0.2, 0.8, size=(views, 90, 64)).astype(np.float32)
+    got = api.dc_gauss_smooth(torch.as_tensor(W, device="cuda"), sigma, radius, adjoint=adjoint)
+    ref = orc.gauss_smooth(W, sigma, radius, adjoint=adjoint)
+    assert rel_l2(got.double().cpu().numpy()[..., :-1], ref[..., :-1]) < 3e-7
